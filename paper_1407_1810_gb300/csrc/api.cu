@@ -132,15 +132,15 @@ int build_metric(pic_ctx *c) {
     row(8)[ii] = rh - rhm;
     row(9)[ii] = 1.0 - sigma_star(d, i, nrg);
     row(10)[ii] = 1.0 - sigma_star(d, i + 0.5, nrg);
-    const double id2n = 2.0 / (rn1 * rn1 - rn * rn), id2h = 2.0 / (rh * rh - rhm * rhm);
+    const double id2n = 2.0 / (rn1 * rn1 - rn * rn);
     row(13)[ii] = hh / rn;
     row(14)[ii] = hh * id2n * rn;
     row(15)[ii] = hh * id2n * rn1;
     row(16)[ii] = hh * id2n * (rn1 - rn);
     row(17)[ii] = dt / rh;
-    row(18)[ii] = dt * id2h * rhm;
-    row(19)[ii] = dt * id2h * rh;
-    row(20)[ii] = dt * id2h * (rh - rhm);
+    row(18)[ii] = dt * rhm;
+    row(19)[ii] = dt * rh;
+    row(20)[ii] = dt * (rh - rhm);
     if (i >= 0 && i <= nrg) {
       double a = std::fmax(i - 0.5, 0.0), b = std::fmin(i + 0.5, (double)nrg);
       row(11)[ii] = 2.0 * M_PI / 3.0 * (std::pow(fr(b), 3) - std::pow(fr(a), 3));
@@ -193,7 +193,7 @@ int build_metric(pic_ctx *c) {
   m.sin_tb = dc(4); m.inv_sin_tb = dc(5); m.inv_dtb = dc(6);
   m.inv_dcos_tb = dc(9); m.vol_t_n = dc(10); m.vol_t_h = dc(11);
   m.bR = dr(13); m.bT0 = dr(14); m.bT1 = dr(15); m.bP = dr(16);
-  m.eR = dr(17); m.eT0 = dr(18); m.eT1 = dr(19); m.eP = dr(20);
+  m.eR = dr(17); m.w0 = dr(18); m.w1 = dr(19); m.wd = dr(20);
   m.cB1 = dc(12); m.cB2 = dc(13); m.cE1 = dc(14); m.cE2 = dc(15); m.cF = dc(16);
   m.cos_tb = dc(17);
   return PIC_OK;
@@ -527,11 +527,23 @@ int pic_create_context(pic_ctx **out, const pic_desc &d, void *stream, int i0, i
   for (int k = 0; k < 6; ++k)
     if ((e = dalloc(&c->f[k], ge))) return fail(e);
   for (int k = 0; k < 3; ++k)
-    if ((e = dalloc(&c->F[k], ge)) || (e = dalloc(&c->Ft[k], ge))) return fail(e);
+    if ((e = dalloc(&c->F[k], ge)) || (e = dalloc(&c->Ft[k], ge)) || (e = dalloc(&c->bh[k], ge))) return fail(e);
   if ((e = dalloc(&c->Q, ge)) || (e = dalloc(&c->Qa, ge)) || (e = dalloc(&c->Qt, ge)) || (e = dalloc(&c->gsnap, ge)))
     return fail(e);
   for (int k = 0; k < 6; ++k) cudaMemset(c->f[k], 0, ge * 8);
-  for (int k = 0; k < 3; ++k) { cudaMemset(c->F[k], 0, ge * 8); cudaMemset(c->Ft[k], 0, ge * 8); }
+  for (int k = 0; k < 3; ++k) {
+    cudaMemset(c->F[k], 0, ge * 8);
+    cudaMemset(c->Ft[k], 0, ge * 8);
+    cudaMemset(c->bh[k], 0, ge * 8);
+  }
+  c->bh_ok = true;  // no field yet
+  if (lossy_first_row(c) >= 0) {  // E of the lossy rows before the layer acts
+    const size_t n = (size_t)(d.nr + 1 - lossy_first_row(c)) * G.LD;
+    for (int k = 0; k < 3; ++k) {
+      if ((e = dalloc(&c->epre[k], n))) return fail(e);
+      cudaMemset(c->epre[k], 0, n * 8);
+    }
+  }
   cudaMemset(c->Q, 0, ge * 8); cudaMemset(c->Qa, 0, ge * 8); cudaMemset(c->Qt, 0, ge * 8);
   cudaMemset(c->gsnap, 0, ge * 8);
   if (d.precision == PIC_FP32) {
@@ -687,32 +699,17 @@ extern "C" int pic_load_particles(pic_ctx *c, int64_t n, const double *x1, const
 void pic_step_body(pic_ctx *c) {
   const double t = c->step * c->G.dt;
   int pr = prof_begin(c, PROF_PARTICLES);
-  if (c->d.precision == PIC_FP64) {
-    for (int k = 0; k < 3; ++k) cudaMemsetAsync(c->F[k], 0, c->grid_elems * 8, c->stream);
-    particles64(c, t);
-    prof_end(c, pr);
-  } else {
-    particles32(c, t);
-    prof_end(c, pr);
-    pr = prof_begin(c, PROF_REDUCE);
-    flux_from_acc(c);
-    prof_end(c, pr);
-  }
-  if (c->d.n_filt > 0) {
-    pr = prof_begin(c, PROF_FILTER);
-    fields_filter(c);
-    prof_end(c, pr);
-  }
+  if (c->d.precision == PIC_FP64) particles64(c, t);
+  else particles32(c, t);
+  prof_end(c, pr);
   pr = prof_begin(c, PROF_FIELDS);
-  fields_b_half(c);
-  fields_e_full(c);
-  fields_b_half(c);
-  fields_finish(c);
+  fields_e_step(c);
+  fields_b_step(c, true);
   prof_end(c, pr);
   c->step += 1;
   if (c->d.inject) {
     pr = prof_begin(c, PROF_INJECT);
-    inject(c, c->step * c->G.dt);
+    inject(c, c->step * c->G.dt, true);
     prof_end(c, pr);
   }
   c->steps_since_sort += 1;
@@ -727,6 +724,7 @@ int pic_prepare_steps(pic_ctx *c, int steps) {
     if (e) return e;
     c->need_sort = false;
   }
+  fields_b_start(c);
   if (!c->have_snap) moments(c, true, nullptr);
   const int64_t need = c->n_used + inject_slots(c) * (int64_t)steps;
   if (c->d.inject && need > c->cap) {
@@ -803,6 +801,7 @@ extern "C" int pic_set_fields(pic_ctx *c, const double *in6, int32_t mem) {
   fields_fill_ghosts(c);
   PIC_CUDA(cudaStreamSynchronize(c->stream));
   cudaFree(tmp);
+  c->bh_ok = false;
   c->have_snap = false;
   return PIC_OK;
 }
@@ -1071,6 +1070,7 @@ int pic_clone_context(pic_ctx *c, pic_ctx **out) {
   for (int q = 0; q < 6; ++q)
     cudaMemcpyAsync(k->f[q], c->f[q], c->grid_elems * 8, cudaMemcpyDeviceToDevice, c->stream);
   fields_fill_ghosts(k);
+  k->bh_ok = false;
   int64_t n = 0;
   if ((e = pic_get_particles(c, &n, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, PIC_MEM_DEVICE)))
     return e;
@@ -1102,7 +1102,7 @@ extern "C" int pic_destroy(pic_ctx *c) {
   cudaFree(c->r_n32);
   cudaFree(c->th_n32);
   cudaFree(c->d_tile_maps);
-  for (int k = 0; k < 3; ++k) { cudaFree(c->F[k]); cudaFree(c->Ft[k]); cudaFree(c->acc[k]); }
+  for (int k = 0; k < 3; ++k) { cudaFree(c->F[k]); cudaFree(c->Ft[k]); cudaFree(c->acc[k]); cudaFree(c->bh[k]); cudaFree(c->epre[k]); }
   cudaFree(c->Q); cudaFree(c->Qa); cudaFree(c->Qt); cudaFree(c->gsnap); cudaFree(c->sig);
   cudaFree(c->d_err); cudaFree(c->d_cnt); cudaFree(c->d_acc);
   cudaFree(c->tiles.start); cudaFree(c->tiles.cursor); cudaFree(c->tiles.bsum);

@@ -146,21 +146,16 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
     if (ctxs[k]->d.inject) max_smooth = std::max(max_smooth, ctxs[k]->d.inject_smooth);
   }
   // the grid phases in launch order, and which members take part in each
-  const int L_FLUX = 0, L_FILT = L_FLUX + 1, L_NODES = L_FILT + max_filt, L_LOSSY = L_NODES + 1,
-            L_GHOSTS = L_LOSSY + 1, L_COPY = L_GHOSTS + 1, L_SIGMA = L_COPY + 1, L_SMOOTH = L_SIGMA + 1,
+  const int L_FLUX = 0, L_FILT = L_FLUX + 1, L_BAND = L_FILT + max_filt, L_SMOOTH = L_BAND + 1,
             L_WRITE = L_SMOOTH + max_smooth, NLISTS = L_WRITE + 1;
   PhaseMaps maps(NLISTS);
   for (int k = 0; k < n; ++k) {
     const pic_ctx *c = ctxs[k];
     maps.add(L_FLUX, k, ens_blocks(c, ENS_FLUX));
     for (int p = 0; p < c->d.n_filt; ++p) maps.add(L_FILT + p, k, ens_blocks(c, ENS_FILTER));
-    maps.add(L_NODES, k, ens_blocks(c, ENS_NODES));
-    maps.add(L_LOSSY, k, ens_blocks(c, ENS_LOSSY));
-    maps.add(L_GHOSTS, k, ens_blocks(c, ENS_GHOSTS));
-    maps.add(L_COPY, k, ens_blocks(c, ENS_COPY32));
+    maps.add(L_BAND, k, ens_blocks(c, ENS_BAND));
     if (c->d.inject) {
-      maps.add(L_SIGMA, k, ens_blocks(c, ENS_SIGMA));
-      for (int p = 0; p < c->d.inject_smooth; ++p) maps.add(L_SMOOTH + p, k, ens_blocks(c, ENS_SIGMA));
+      for (int p = 0; p < c->d.inject_smooth; ++p) maps.add(L_SMOOTH + p, k, ens_blocks(c, ENS_SMOOTH));
       maps.add(L_WRITE, k, ens_blocks(c, ENS_WRITE));
     }
   }
@@ -193,6 +188,9 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
     cudaError_t ce = cudaStreamSynchronize(ctxs[k]->stream);  // earlier work of each member first
     if (ce != cudaSuccess) err = pic_cuda_check(ce, "ensemble member stream");
   }
+  int64_t particles = 0;
+  for (int k = 0; k < n; ++k) particles += ctxs[k]->n_used;
+  for (int k = 0; k < n; ++k) ctxs[k]->ens_particles = particles;
   std::vector<StepTiles> tiles(ENS_MAX_BLOCK);
   std::vector<pic_ctx *> due;
   EnsSortScratch sort_scratch;
@@ -232,8 +230,8 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
           ++c->launches;
         }
         ens_fill_field_arg(c, &fa[k]);
-        c->launches += 1 + 3 * (int64_t)c->d.n_filt + 3 + (ens_blocks(c, ENS_LOSSY) > 0) + 2;
-        if (c->d.n_filt & 1)
+        c->launches += grid_launches(c);
+        if (filter_swaps(c))
           for (int q = 0; q < 3; ++q) std::swap(c->F[q], c->Ft[q]);
         c->step += 1;
         if (c->d.inject) {
@@ -241,7 +239,6 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
           fa[k].inj_base = c->n_used;
           fa[k].inj_id0 = c->next_id;
           fa[k].inj_step = (uint64_t)c->step;
-          c->launches += 2 + c->d.inject_smooth;
           const int64_t nslots = (int64_t)G.nth * c->d.pairs_per_cell * 2;
           c->n_used += nslots;
           c->next_id += nslots;
@@ -265,24 +262,16 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
         for (int kind = 0; kind < ENS_TILE_KINDS; ++kind)
           if (!T.blocks[kind].empty())
             nodes += ens_tiles32(kind, T.arg[kind].data(), T.blocks[kind].data(), (int)T.blocks[kind].size(), origin);
-        ens_flux_from_acc(dfa, L(L_FLUX), maps.blocks(L_FLUX), origin), ++nodes;
+        if (maps.blocks(L_FLUX) > 0) ens_flux(dfa, L(L_FLUX), maps.blocks(L_FLUX), origin), ++nodes;
         for (int p = 0; p < max_filt; ++p)
           if (maps.blocks(L_FILT + p) > 0) ens_filter(dfa, L(L_FILT + p), maps.blocks(L_FILT + p), p, origin), ++nodes;
-        ens_b_half(dfa, L(L_NODES), maps.blocks(L_NODES), origin);
-        ens_e_full(dfa, L(L_NODES), maps.blocks(L_NODES), origin);
-        ens_b_half(dfa, L(L_NODES), maps.blocks(L_NODES), origin);
-        nodes += 3;
-        if (maps.blocks(L_LOSSY) > 0) ens_lossy(dfa, L(L_LOSSY), maps.blocks(L_LOSSY), origin), ++nodes;
-        ens_ghosts(dfa, L(L_GHOSTS), maps.blocks(L_GHOSTS), origin);
-        ens_copy32(dfa, L(L_COPY), maps.blocks(L_COPY), origin);
+        ens_e_step(dfa, L(L_BAND), maps.blocks(L_BAND), origin);
+        ens_b_step(dfa, L(L_BAND), maps.blocks(L_BAND), origin);
         nodes += 2;
-        if (maps.blocks(L_SIGMA) > 0) {
-          ens_inject_sigma(dfa, L(L_SIGMA), maps.blocks(L_SIGMA), origin), ++nodes;
-          for (int p = 0; p < max_smooth; ++p)
-            if (maps.blocks(L_SMOOTH + p) > 0)
-              ens_inject_smooth(dfa, L(L_SMOOTH + p), maps.blocks(L_SMOOTH + p), p, origin), ++nodes;
-          ens_inject_write(dfa, L(L_WRITE), maps.blocks(L_WRITE), origin), ++nodes;
-        }
+        for (int p = 0; p < max_smooth; ++p)
+          if (maps.blocks(L_SMOOTH + p) > 0)
+            ens_inject_smooth(dfa, L(L_SMOOTH + p), maps.blocks(L_SMOOTH + p), p, origin), ++nodes;
+        if (maps.blocks(L_WRITE) > 0) ens_inject_write(dfa, L(L_WRITE), maps.blocks(L_WRITE), origin), ++nodes;
       }
       cudaError_t ce2 = cudaStreamEndCapture(origin, &graph);
       if (ce == cudaSuccess) ce = ce2;
@@ -321,6 +310,7 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
     // the staging table is refilled next: its copy must have completed
     if (!err) cudaEventSynchronize(after);
   }
+  for (int k = 0; k < n; ++k) ctxs[k]->ens_particles = 0;
   if (origin) cudaStreamSynchronize(origin);
   if (exec) cudaGraphExecDestroy(exec);
   if (after) cudaEventDestroy(after);

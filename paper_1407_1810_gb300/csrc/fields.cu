@@ -20,84 +20,147 @@ constexpr int BX = 32, BY = 8;
 
 inline dim3 grid2(int ni, int nj) { return dim3((nj + BX - 1) / BX, (ni + BY - 1) / BY); }
 
-// B <- B - h c curl E over the faces of the primary grid (first three lines of
-// Eq. discreteeq).  One thread per node (i, j), 0 <= i <= nr, 0 <= j <= nth.
-// (the factors of dt / 2 and the metric are folded into the row and column
-// coefficient tables of Metric: a few FP64 FMAs per node, the rate that
-// limits this kernel)
-__device__ __forceinline__ void b_half_node(const Grid &G, int i, int j, const double *__restrict__ Er,
-                                            const double *__restrict__ Et, const double *__restrict__ Ep,
-                                            double *__restrict__ Br, double *__restrict__ Bt,
-                                            double *__restrict__ Bp) {
-  if (i > G.nr || j > G.nth) return;
-  const Metric &m = G.m;
-  const int ri = i + G.PI, cj = j + G.PJ;
-  const size_t o = gidx(G, i, j);
-  if (j < G.nth)  // B_r at (i, j+1/2)
-    Br[o] += m.bR[ri] * (Ep[o] * m.cB1[cj] - Ep[o + 1] * m.cB2[cj]);
-  if (i < G.nr) {
-    const double t0 = m.bT0[ri], t1 = m.bT1[ri];
-    if (j >= 1 && j < G.nth)  // B_th at (i+1/2, j); zero on the axis
-      Bt[o] += t1 * Ep[o + G.LD] - t0 * Ep[o];
-    if (j < G.nth)  // B_ph at (i+1/2, j+1/2)
-      Bp[o] += (t0 * Et[o] - t1 * Et[o + G.LD]) - (Er[o] - Er[o + 1]) * (m.bP[ri] * m.inv_dth_t[cj]);
-  }
-}
+// ---- the leapfrog of a step ---------------------------------------------------
+// A step takes B forward by a half step, E by a full one and B by a half
+// again (App. A).  The second half of one step and the first half of the next
+// add the same curl of the same E, so the B update below forms it once, adds
+// it to B^{n+1/2} for the B at integer time that the gather and every reader
+// use (f[BR..BPH]), and adds it again for the half-step B of the next step
+// (bh).  bh is always B + dB(E) of the stored fields: fields_b_start forms it
+// after the fields were replaced.  Only the lossy rows take the curl twice
+// (the layer scales E and B between the two halves).
+//
+// The FP64 pipe bounds these kernels (2 lanes a clock and SM): their cost is
+// the number of FP64 operations a node, 31 here against 46 for three passes
+// and FP64 -> FP32 conversion instructions.  The operations are explicitly
+// rounded: single-context, batched and slab kernels give the same bits.
 
-__global__ void k_b_half(Grid G, const double *__restrict__ Er, const double *__restrict__ Et,
-                         const double *__restrict__ Ep, double *__restrict__ Br, double *__restrict__ Bt,
-                         double *__restrict__ Bp) {
-  b_half_node(G, blockIdx.y * BY + threadIdx.y, blockIdx.x * BX + threadIdx.x, Er, Et, Ep, Br, Bt, Bp);
+// h c curl E at node (i, j) for the three components of B (h = dt / 2)
+__device__ __forceinline__ void curl_e(const Metric &m, int ri, int cj, double er, double er_j, double et,
+                                       double et_i, double ep, double ep_j, double ep_i, double d[3]) {
+  const double t0 = m.bT0[ri], t1 = m.bT1[ri];
+  d[0] = __dmul_rn(m.bR[ri], __fma_rn(ep, m.cB1[cj], -__dmul_rn(ep_j, m.cB2[cj])));
+  d[1] = __fma_rn(t1, ep_i, -__dmul_rn(t0, ep));
+  d[2] = __fma_rn(-__dmul_rn(m.bP[ri], m.inv_dth_t[cj]), __dsub_rn(er, er_j), __fma_rn(t0, et, -__dmul_rn(t1, et_i)));
 }
 
 // E <- E + dt c curl B - F / dA over the faces of the dual grid (last three
 // lines of Eq. discreteeq; E_r on the axis by Eq. erpolarupdate, obtained here
 // from the same formula with sin(tb_{-1}) = sin(tb_{nth}) = 0 and the cap
-// areas in inv_dcos_tb).  E_th, E_ph stay 0 on the conductors (i = 0, nr) and
-// E_ph on the axis.
-__device__ __forceinline__ void e_full_node(const Grid &G, int i, int j, double *__restrict__ Er,
-                                            double *__restrict__ Et, double *__restrict__ Ep,
-                                            const double *__restrict__ Br, const double *__restrict__ Bt,
-                                            const double *__restrict__ Bp, const double *__restrict__ Fr,
-                                            const double *__restrict__ Ft, const double *__restrict__ Fp) {
-  if (i > G.nr || j > G.nth) return;
+// areas in inv_dcos_tb), then the lossy layer (Eq. EBcond: times 1 - sigma*
+// at the component's own radial stagger), whose rows keep the E before it in
+// epre for the second half step of B.  E_th, E_ph stay 0 on the conductors
+// (i = 0, nr) and E_ph on the axis.
+__device__ __forceinline__ void e_node(const EnsFieldArg &S, int i, int j, double Fr, double Ft, double Fp) {
+  const Grid &G = S.G;
   const Metric &m = G.m;
   const int ri = i + G.PI, cj = j + G.PJ;
   const size_t o = gidx(G, i, j);
-  if (i < G.nr)  // E_r at (i+1/2, j)
-    Er[o] += m.eR[ri] * (Bp[o] * m.cE1[cj] - Bp[o - 1] * m.cE2[cj]) - Fr[o] * (m.inv_area_h[ri] * m.inv_dcos_tb[cj]);
+  const double *Br = S.bh[0], *Bt = S.bh[1], *Bp = S.bh[2];
+  const bool lossy = S.lossy_i0 >= 0 && i >= S.lossy_i0;
+  const size_t l = lossy ? (size_t)(i - S.lossy_i0) * G.LD + cj : 0;
+  if (i < G.nr) {  // E_r at (i+1/2, j)
+    const double c = __fma_rn(Bp[o], m.cE1[cj], -__dmul_rn(Bp[o - 1], m.cE2[cj]));
+    double e = __fma_rn(m.eR[ri], c, S.f[ER][o]);
+    e = __fma_rn(-Fr, __dmul_rn(m.inv_area_h[ri], m.inv_dcos_tb[cj]), e);
+    if (lossy) { S.epre[0][l] = e; e = __dmul_rn(e, m.keep_h[ri]); }
+    S.f[ER][o] = e;
+  }
   // E_th, E_ph stay 0 on a conductor; a slab's open side is an interior row
-  if ((i >= 1 || G.open_lo) && (i < G.nr || G.open_hi)) {
-    const double t0 = m.eT0[ri], t1 = m.eT1[ri], id2 = m.inv_dr2_h[ri];
-    if (j < G.nth)  // E_th at (i, j+1/2)
-      Et[o] += (t0 * Bp[o - G.LD] - t1 * Bp[o]) - Ft[o] * (m.cF[cj] * id2);
-    if (j >= 1 && j < G.nth) {  // E_ph at (i, j)
-      const double idt = m.inv_dtb[cj];
-      Ep[o] += ((t1 * Bt[o] - t0 * Bt[o - G.LD]) - (Br[o] - Br[o - 1]) * (m.eP[ri] * idt)) - Fp[o] * (idt * id2);
-    }
+  const bool in = (i >= 1 || G.open_lo) && (i < G.nr || G.open_hi);
+  const double w0 = m.w0[ri], w1 = m.w1[ri], id2 = m.inv_dr2_h[ri];
+  if (in && j < G.nth) {  // E_th at (i, j+1/2)
+    const double c = __fma_rn(-m.cF[cj], Ft, __fma_rn(w0, Bp[o - G.LD], -__dmul_rn(w1, Bp[o])));
+    double e = __fma_rn(id2, c, S.f[ETH][o]);
+    if (lossy) { S.epre[1][l] = e; e = __dmul_rn(e, m.keep_n[ri]); }
+    S.f[ETH][o] = e;
+  }
+  if (in && j >= 1 && j < G.nth) {  // E_ph at (i, j)
+    const double c = __fma_rn(m.wd[ri], __dsub_rn(Br[o], Br[o - 1]), Fp);
+    const double k = __fma_rn(-m.inv_dtb[cj], c, __fma_rn(w1, Bt[o], -__dmul_rn(w0, Bt[o - G.LD])));
+    double e = __fma_rn(id2, k, S.f[EPH][o]);
+    if (lossy) { S.epre[2][l] = e; e = __dmul_rn(e, m.keep_n[ri]); }
+    S.f[EPH][o] = e;
   }
 }
 
-__global__ void k_e_full(Grid G, double *__restrict__ Er, double *__restrict__ Et, double *__restrict__ Ep,
-                         const double *__restrict__ Br, const double *__restrict__ Bt,
-                         const double *__restrict__ Bp, const double *__restrict__ Fr,
-                         const double *__restrict__ Ft, const double *__restrict__ Fp) {
-  e_full_node(G, blockIdx.y * BY + threadIdx.y, blockIdx.x * BX + threadIdx.x, Er, Et, Ep, Br, Bt, Bp, Fr, Ft, Fp);
-}
-
-// Lossy layer, Eq. (EBcond): every component times 1 - sigma* at its own
-// radial stagger, rows i0..nr.
-__device__ __forceinline__ void lossy_node(const Grid &G, int i, int j, double *Er, double *Et, double *Ep,
-                                           double *Br, double *Bt, double *Bp) {
-  if (i > G.nr || j > G.nth) return;
+// B at integer time and at the next half step of node (i, j), the axis
+// continuation of the half-integer-j components into columns -1 and nth (B_r
+// even; E_th, B_ph odd) and the FP32 gather copies of the six components.
+// SIGMA: the row at the star also forms the injection's surface charge.
+template <bool FP32>
+__device__ __forceinline__ void b_node(const EnsFieldArg &S, int i, int j) {
+  const Grid &G = S.G;
+  const Metric &m = G.m;
+  const int ri = i + G.PI, cj = j + G.PJ;
   const size_t o = gidx(G, i, j);
-  const double kn = G.m.keep_n[i + G.PI], kh = G.m.keep_h[i + G.PI];
-  Er[o] *= kh; Bt[o] *= kh; Bp[o] *= kh;
-  Et[o] *= kn; Ep[o] *= kn; Br[o] *= kn;
+  const double er = S.f[ER][o], er_j = S.f[ER][o + 1], et = S.f[ETH][o], et_i = S.f[ETH][o + G.LD];
+  const double ep = S.f[EPH][o], ep_j = S.f[EPH][o + 1], ep_i = S.f[EPH][o + G.LD];
+  double d[3], d2[3], b[3];
+  curl_e(m, ri, cj, er, er_j, et, et_i, ep, ep_j, ep_i, d2);
+  const bool lossy = S.lossy_i0 >= 0 && i >= S.lossy_i0;
+  if (lossy) {  // the half step before the layer: E as it was then
+    const size_t l = (size_t)(i - S.lossy_i0) * G.LD + cj;
+    const bool up = i < G.nr;
+    curl_e(m, ri, cj, S.epre[0][l], S.epre[0][l + 1], S.epre[1][l], up ? S.epre[1][l + G.LD] : 0.0, S.epre[2][l],
+           S.epre[2][l + 1], up ? S.epre[2][l + G.LD] : 0.0, d);
+  } else {
+    d[0] = d2[0]; d[1] = d2[1]; d[2] = d2[2];
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) b[k] = __dadd_rn(S.bh[k][o], d[k]);
+  if (lossy) {
+    b[0] = __dmul_rn(b[0], m.keep_n[ri]);
+    b[1] = __dmul_rn(b[1], m.keep_h[ri]);
+    b[2] = __dmul_rn(b[2], m.keep_h[ri]);
+  }
+  const bool hj = j < G.nth, hi = i < G.nr;  // half-integer columns / rows of the grid
+  if (hj) {  // B_r at (i, j+1/2)
+    S.f[BR][o] = b[0];
+    S.bh[0][o] = __dadd_rn(b[0], d2[0]);
+  }
+  if (hi && j >= 1 && hj) {  // B_th at (i+1/2, j); zero on the axis
+    S.f[BTH][o] = b[1];
+    S.bh[1][o] = __dadd_rn(b[1], d2[1]);
+  } else {
+    b[1] = 0.0;
+  }
+  if (hi && hj) {  // B_ph at (i+1/2, j+1/2)
+    S.f[BPH][o] = b[2];
+    S.bh[2][o] = __dadd_rn(b[2], d2[2]);
+  } else {
+    b[2] = 0.0;
+  }
+  float q[6];
+  if (FP32) {
+    q[0] = f64_to_f32(er); q[1] = f64_to_f32(et); q[2] = f64_to_f32(ep);
+    q[3] = f64_to_f32(b[0]); q[4] = f64_to_f32(b[1]); q[5] = f64_to_f32(b[2]);
+    S.f32[ER][o] = q[0]; S.f32[EPH][o] = q[2]; S.f32[BTH][o] = q[4];
+    if (hj) { S.f32[ETH][o] = q[1]; S.f32[BR][o] = q[3]; S.f32[BPH][o] = q[5]; }
+  }
+  if (j == 0 || j == G.nth - 1) {
+    const size_t a = j == 0 ? o - 1 : o + 1;
+    S.f[ETH][a] = -et; S.f[BR][a] = b[0]; S.f[BPH][a] = -b[2];
+    if (FP32) { S.f32[ETH][a] = -q[1]; S.f32[BR][a] = q[3]; S.f32[BPH][a] = -q[5]; }
+  }
 }
 
-__global__ void k_lossy(Grid G, double *Er, double *Et, double *Ep, double *Br, double *Bt, double *Bp, int i0) {
-  lossy_node(G, i0 + blockIdx.y * BY + threadIdx.y, blockIdx.x * BX + threadIdx.x, Er, Et, Ep, Br, Bt, Bp);
+// bh = B + dB(E) of the stored fields at node (i, j)
+__device__ __forceinline__ void b_start_node(const EnsFieldArg &S, int i, int j) {
+  const Grid &G = S.G;
+  const size_t o = gidx(G, i, j);
+  double d[3];
+  curl_e(G.m, i + G.PI, j + G.PJ, S.f[ER][o], S.f[ER][o + 1], S.f[ETH][o], S.f[ETH][o + G.LD], S.f[EPH][o],
+         S.f[EPH][o + 1], S.f[EPH][o + G.LD], d);
+  const bool hj = j < G.nth, hi = i < G.nr;
+  if (hj) S.bh[0][o] = __dadd_rn(S.f[BR][o], d[0]);
+  if (hi && j >= 1 && hj) S.bh[1][o] = __dadd_rn(S.f[BTH][o], d[1]);
+  if (hi && hj) S.bh[2][o] = __dadd_rn(S.f[BPH][o], d[2]);
+}
+
+__global__ void k_b_start(const __grid_constant__ EnsFieldArg S) {
+  const int i = blockIdx.y * BY + threadIdx.y, j = blockIdx.x * BX + threadIdx.x;
+  if (i <= S.G.nr && j <= S.G.nth) b_start_node(S, i, j);
 }
 
 // Axisymmetric continuation of the half-integer-j components into columns -1
@@ -125,8 +188,8 @@ __device__ __forceinline__ void copy32_node(const Grid &G, int i, int j, const d
                                             float *b3, float *b4, float *b5) {
   if (i > G.nr + G.g || j > G.nth) return;
   const size_t k = gidx(G, i, j);
-  b0[k] = (float)a0[k]; b1[k] = (float)a1[k]; b2[k] = (float)a2[k];
-  b3[k] = (float)a3[k]; b4[k] = (float)a4[k]; b5[k] = (float)a5[k];
+  b0[k] = f64_to_f32(a0[k]); b1[k] = f64_to_f32(a1[k]); b2[k] = f64_to_f32(a2[k]);
+  b3[k] = f64_to_f32(a3[k]); b4[k] = f64_to_f32(a4[k]); b5[k] = f64_to_f32(a5[k]);
 }
 
 __global__ void k_copy32(Grid G, const double *__restrict__ a0, const double *__restrict__ a1,
@@ -193,6 +256,224 @@ __device__ __forceinline__ void sigma_cell(const Grid &G, int j, const double *_
   const double s = 0.5 * (e[0] + e[1]);
   sig[j] = s;
   if (smax) atomicMax(smax, __double_as_longlong(fabs(s)));
+}
+
+// ---- deposit -> filtered flux, in one pass ----------------------------------
+// The N passes of the 1-2-1 filter act along rows and columns independently,
+// so they are one convolution with the 2N + 1 binomial weights along each,
+// taken from a shared-memory tile with a halo of N nodes:
+//  - the polar fold of App. B (a pass's share that lands beyond the axis comes
+//    back to its mirror point) equals the plain convolution of the deposit
+//    continued past the pole as its mirror image -- even, with the pole node
+//    doubled and its result halved, for integer j; odd for half-integer j;
+//  - rows that leave the ghost band are dropped after every pass: the
+//    convolution of the deposit continued as an odd image past row -g - 1 and
+//    nr + g + 1.
+// The weights are integers over 4^N a direction, so the FP32 path's fixed-point
+// sums are filtered exactly in 64-bit integers, on the pipes that have the
+// room, and rounded once (a nine-launch FP64 filter took 255 us of a 1024^2
+// rotator step, the FP64 pipe 86 % busy).  A tile whose sums leave no room for
+// the 16^N of the weights takes 128-bit integers: the same exact result.
+constexpr int FUSE_FILT = 4;  // passes the tile's halo holds; more run pass by pass
+constexpr int TW = BX + 2 * FUSE_FILT, TH = BY + 2 * FUSE_FILT;
+__constant__ int FILT_W[FUSE_FILT + 1][FUSE_FILT + 1] = {  // C(2N, N + k)
+    {1, 0, 0, 0, 0}, {2, 1, 0, 0, 0}, {6, 4, 1, 0, 0}, {20, 15, 6, 1, 0}, {70, 56, 28, 8, 1}};
+
+// Images of a tile's rows and columns, formed once per block: array offset (or
+// -1: zero) and factor (+-1, +-2) of row i0 - N + r and, for integer and
+// half-integer j, of column j0 - N + q of the continued deposit.
+struct FiltImages {
+  int row[TH], col[2][TW];
+  signed char row_c[TH], col_c[2][TW];
+};
+
+__device__ __forceinline__ void filt_images(FiltImages &im, const Grid &G, int i0, int j0, int N) {
+  const int t = threadIdx.y * BX + threadIdx.x;
+  if (t < BY + 2 * N) {
+    const int lo = -G.g - 1, hi = G.nr + G.g + 1;
+    int ii = i0 - N + t, c = 1;
+    if (ii <= lo) { ii = 2 * lo - ii; c = -1; }
+    else if (ii >= hi) { ii = 2 * hi - ii; c = -1; }
+    im.row[t] = ii <= lo || ii >= hi ? -1 : ii + G.PI;  // -1: the dropped row itself
+    im.row_c[t] = (signed char)c;
+  }
+  const int u = t - 64, n = G.nth;  // other warps than the rows'
+  if (u >= 0 && u < 2 * TW) {
+    const int half = u / TW, q = u % TW;
+    int jj = j0 - N + q, c = 1;
+    if (jj > n + 2 * FUSE_FILT) jj = n;  // right of every column that a node of the tile reads
+    if (half) {
+      while (jj < 0 || jj >= n) { jj = jj < 0 ? -1 - jj : 2 * n - 1 - jj; c = -c; }
+    } else {
+      while (jj < 0 || jj > n) jj = jj < 0 ? -jj : 2 * n - jj;
+      if (jj == 0 || jj == n) c = 2;
+    }
+    im.col[half][q] = jj + G.PJ;
+    im.col_c[half][q] = (signed char)c;
+  }
+  __syncthreads();
+}
+
+template <class T, int NC>
+struct FiltTile {
+  T in[NC][TH][TW + 1];
+  T mid[NC][TH][BX + 1];
+};
+
+// NC components (the first of them component c0) of the tile with N passes at
+// this thread's node; every thread of the block calls it
+template <class T, int NC, class L>
+__device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &im, const Grid &G, int N, int c0,
+                                          T out[NC], const L &load) {
+  const int tx = threadIdx.x, ty = threadIdx.y, w = BX + 2 * N, h = BY + 2 * N;
+#pragma unroll
+  for (int k = 0; k < NC; ++k)
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const int r = ty + a * BY, q = tx + b * BX, half = c0 + k == 1;
+        if (r < h && q < w) {
+          const int ro = im.row[r];
+          t.in[k][r][q] = ro < 0 ? T(0)
+                                 : T(im.row_c[r] * im.col_c[half][q]) *
+                                       load(c0 + k, (size_t)ro * G.LD + im.col[half][q]);
+        }
+      }
+  __syncthreads();
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int r = ty + a * BY;
+    if (r < h)
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const T *x = &t.in[k][r][tx + N];
+        T s = T(FILT_W[N][0]) * x[0];
+        for (int m = 1; m <= N; ++m) s += T(FILT_W[N][m]) * (x[-m] + x[m]);
+        t.mid[k][r][tx] = s;
+      }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    T s = T(FILT_W[N][0]) * t.mid[k][ty + N][tx];
+    for (int m = 1; m <= N; ++m) s += T(FILT_W[N][m]) * (t.mid[k][ty + N - m][tx] + t.mid[k][ty + N + m][tx]);
+    out[k] = s;
+  }
+}
+
+struct FiltSmem {
+  FiltImages im;
+  union {
+    FiltTile<long long, 3> q;
+    FiltTile<__int128, 1> w;
+    FiltTile<double, 3> d;
+  };
+  __device__ FiltSmem() {}
+};
+
+// One block (32 x 8 nodes of the ghost band -g..nr+g, 0..nth) of the E update:
+// the flux of the deposit filtered and stored (the step's fluxes), then E.
+template <bool FP32>
+__device__ __forceinline__ void e_block(const EnsFieldArg &S, unsigned b, FiltSmem &sm) {
+  const Grid &G = S.G;
+  const unsigned gx = (unsigned)(G.nth + 1 + BX - 1) / BX;
+  const int i0 = -G.g + (int)(b / gx) * BY, j0 = (int)(b % gx) * BX;
+  const int i = i0 + (int)threadIdx.y, j = j0 + (int)threadIdx.x;
+  const bool in = i <= G.nr + G.g && j <= G.nth;
+  const size_t o = in ? gidx(G, i, j) : 0;
+  const int N = S.n_filt;
+  const bool pole = j == 0 || j == G.nth;
+  double F[3] = {0.0, 0.0, 0.0};
+  if (N > FUSE_FILT) {  // filtered pass by pass before this launch
+    if (in)
+      for (int k = 0; k < 3; ++k) F[k] = S.Fout[k][o];
+  } else if (FP32) {
+    const int s = qexp_value(S.qexp) - KFIX;  // one flux unit is 2^s of charge
+    if (N == 0) {
+      if (in)
+        for (int k = 0; k < 3; ++k) F[k] = fixed_to_f64(S.acc[k][o], s);
+    } else {
+      const long long lim = 1ll << (60 - 4 * N);
+      bool big = false;
+      long long v[3];
+      filt_images(sm.im, G, i0, j0, N);
+      filt_conv(sm.q, sm.im, G, N, 0, v, [&](int k, size_t x) {
+        const long long y = S.acc[k][x];
+        big |= y >= lim || y <= -lim;
+        return y;
+      });
+#pragma unroll
+      for (int k = 0; k < 3; ++k) F[k] = fixed_to_f64(k != 1 && pole ? v[k] / 2 : v[k], s - 4 * N);
+      if (__syncthreads_or(big)) {
+        for (int k = 0; k < 3; ++k) {
+          __int128 z[1];
+          filt_conv(sm.w, sm.im, G, N, k, z, [&](int c, size_t x) { return (__int128)S.acc[c][x]; });
+          F[k] = fixed_to_f64(k != 1 && pole ? z[0] / 2 : z[0], s - 4 * N);
+          __syncthreads();
+        }
+      }
+    }
+  } else {
+    if (N == 0) {
+      if (in)
+        for (int k = 0; k < 3; ++k) F[k] = S.Fin[k][o];
+    } else {
+      const double sc = __longlong_as_double((long long)(1023 - 4 * N) << 52);  // 16^-N
+      double v[3];
+      filt_images(sm.im, G, i0, j0, N);
+      filt_conv(sm.d, sm.im, G, N, 0, v, [&](int k, size_t x) { return S.Fin[k][x]; });
+#pragma unroll
+      for (int k = 0; k < 3; ++k) F[k] = v[k] * (k != 1 && pole ? 0.5 * sc : sc);
+    }
+  }
+  if (b == 0 && threadIdx.x == 0 && threadIdx.y == 0 && S.inject) S.cnt[CNT_SMAX] = 0;  // raised by the B update
+  if (!in) return;
+  if (N <= FUSE_FILT) {
+    S.Fout[0][o] = F[0];
+    if (j < G.nth) S.Fout[1][o] = F[1];
+    S.Fout[2][o] = F[2];
+  }
+  if (i >= 0 && i <= G.nr) e_node(S, i, j, F[0], F[1], F[2]);
+}
+
+// One block of the B update over the same nodes; it also clears the deposit
+// of the step, and with `sigma` forms the surface charge of the injection
+// from the new E_r (its maximum too, when no smoothing pass follows).
+template <bool FP32>
+__device__ __forceinline__ void b_block(const EnsFieldArg &S, unsigned b, bool sigma) {
+  const Grid &G = S.G;
+  const unsigned gx = (unsigned)(G.nth + 1 + BX - 1) / BX;
+  const int i = -G.g + (int)((b / gx) * BY + threadIdx.y), j = (int)((b % gx) * BX + threadIdx.x);
+  if (i > G.nr + G.g || j > G.nth) return;
+  const size_t o = gidx(G, i, j);
+  if (FP32)
+    for (int k = 0; k < 3; ++k) S.acc[k][o] = 0;
+  else  // (an even number of separate passes leaves the filtered flux in Fin)
+    for (int k = 0; k < 3; ++k) (S.Fout[k] == S.Fin[k] ? S.Ftmp : S.Fin)[k][o] = 0.0;
+  if (i < 0 || i > G.nr) return;
+  b_node<FP32>(S, i, j);
+  if (sigma && i == 0) sigma_cell(G, j, S.f[ER], S.t_inj, S.sig, S.inject_smooth ? nullptr : S.cnt + CNT_SMAX);
+}
+
+template <bool FP32>
+__global__ void __launch_bounds__(BX *BY) k_e_step(const __grid_constant__ EnsFieldArg S) {
+  __shared__ FiltSmem sm;
+  e_block<FP32>(S, blockIdx.x, sm);
+}
+template <bool FP32>
+__global__ void __launch_bounds__(BX *BY) k_b_step(const __grid_constant__ EnsFieldArg S, int sigma) {
+  b_block<FP32>(S, blockIdx.x, sigma != 0);
+}
+
+// fixed point -> FP64 fluxes over the ghost band, for the pass-by-pass filter
+__global__ void k_flux_from_acc(const __grid_constant__ EnsFieldArg S) {
+  const Grid &G = S.G;
+  const int i = -G.g + (int)(blockIdx.y * BY + threadIdx.y), j = blockIdx.x * BX + threadIdx.x;
+  if (i > G.nr + G.g || j > G.nth) return;
+  const int s = qexp_value(S.qexp) - KFIX;
+  const size_t o = gidx(G, i, j);
+  for (int k = 0; k < 3; ++k) S.Fin[k][o] = fixed_to_f64(S.acc[k][o], s);
 }
 
 __global__ void k_inject_sigma(Grid G, const double *__restrict__ Er, double t, double *sig, long long *smax) {
@@ -393,55 +674,48 @@ __global__ void k_ens_filter(const EnsFieldArg *__restrict__ tab, EnsList L, int
   filter_node(G, n.i, n.j, in, out, comp == 1);
 }
 
-__global__ void k_ens_b_half(const EnsFieldArg *__restrict__ tab, EnsList L) {
+__global__ void k_ens_flux(const EnsFieldArg *__restrict__ tab, EnsList L) {
   const int2 e = L.blk[blockIdx.x];
   const EnsFieldArg &E = tab[e.x];
-  const Node2 n = node_of((unsigned)e.y, E.G.nth + 1, 0);
-  b_half_node(E.G, n.i, n.j, E.f[ER], E.f[ETH], E.f[EPH], E.f[BR], E.f[BTH], E.f[BPH]);
+  const Node2 n = node_of((unsigned)e.y, E.G.nth + 1, -E.G.g);
+  if (n.i > E.G.nr + E.G.g || n.j > E.G.nth) return;
+  const int s = qexp_value(E.qexp) - KFIX;
+  const size_t o = gidx(E.G, n.i, n.j);
+  for (int k = 0; k < 3; ++k) E.Fin[k][o] = fixed_to_f64(E.acc[k][o], s);
 }
 
-__global__ void k_ens_e_full(const EnsFieldArg *__restrict__ tab, EnsList L) {
+// the member of this block, its argument copied to shared memory (one
+// coalesced load instead of a dependent load for every array and table)
+__device__ __forceinline__ unsigned ens_member(const EnsFieldArg *__restrict__ tab, const EnsList &L,
+                                               EnsFieldArg &S) {
+  static_assert(sizeof(EnsFieldArg) % 8 == 0 && sizeof(EnsFieldArg) <= 8 * BX * BY, "copied by one block");
   const int2 e = L.blk[blockIdx.x];
-  const EnsFieldArg &E = tab[e.x];
-  const Node2 n = node_of((unsigned)e.y, E.G.nth + 1, 0);
-  e_full_node(E.G, n.i, n.j, E.f[ER], E.f[ETH], E.f[EPH], E.f[BR], E.f[BTH], E.f[BPH], E.Fout[0], E.Fout[1],
-              E.Fout[2]);
+  const int t = threadIdx.y * BX + threadIdx.x;
+  if (t < (int)(sizeof(EnsFieldArg) / 8))
+    reinterpret_cast<unsigned long long *>(&S)[t] = reinterpret_cast<const unsigned long long *>(tab + e.x)[t];
+  __syncthreads();
+  return (unsigned)e.y;
+}
+struct EnsMember {
+  EnsFieldArg S;
+  __device__ EnsMember() {}
+};
+
+__global__ void __launch_bounds__(BX *BY) k_ens_e_step(const EnsFieldArg *__restrict__ tab, EnsList L) {
+  __shared__ FiltSmem sm;
+  __shared__ EnsMember M;
+  const unsigned b = ens_member(tab, L, M.S);
+  e_block<true>(M.S, b, sm);
 }
 
-__global__ void k_ens_lossy(const EnsFieldArg *__restrict__ tab, EnsList L) {
-  const int2 e = L.blk[blockIdx.x];
-  const EnsFieldArg &E = tab[e.x];
-  const Node2 n = node_of((unsigned)e.y, E.G.nth + 1, E.lossy_i0);
-  lossy_node(E.G, n.i, n.j, E.f[0], E.f[1], E.f[2], E.f[3], E.f[4], E.f[5]);
-}
-
-// axis ghosts; block 0 of a member that injects also clears the surface
-// charge maximum its injection will raise later in the step
-__global__ void k_ens_ghosts(const EnsFieldArg *__restrict__ tab, EnsList L) {
-  const int2 e = L.blk[blockIdx.x];
-  const EnsFieldArg &E = tab[e.x];
-  const unsigned b = (unsigned)e.y;
-  if (b == 0 && threadIdx.x == 0 && E.inject) E.cnt[CNT_SMAX] = 0;
-  ghost_row(E.G, (int)(b * blockDim.x + threadIdx.x), E.f[ETH], E.f[BR], E.f[BPH]);
-}
-
-__global__ void k_ens_copy32(const EnsFieldArg *__restrict__ tab, EnsList L) {
-  const int2 e = L.blk[blockIdx.x];
-  const EnsFieldArg &E = tab[e.x];
-  const Node2 n = node_of((unsigned)e.y, E.G.nth + 2, -E.G.g);
-  copy32_node(E.G, n.i, n.j - 1, E.f[0], E.f[1], E.f[2], E.f[3], E.f[4], E.f[5], E.f32[0], E.f32[1], E.f32[2],
-              E.f32[3], E.f32[4], E.f32[5]);
+__global__ void __launch_bounds__(BX *BY) k_ens_b_step(const EnsFieldArg *__restrict__ tab, EnsList L) {
+  __shared__ EnsMember M;
+  const unsigned b = ens_member(tab, L, M.S);
+  b_block<true>(M.S, b, M.S.inject != 0);
 }
 
 __device__ inline InjectRule ens_rule(const EnsFieldArg &E) {
   return InjectRule{E.inject, E.npp, E.f_inj, E.inject_q, E.inject_seed, E.inj_step};
-}
-
-__global__ void k_ens_sigma(const EnsFieldArg *__restrict__ tab, EnsList L) {
-  const int2 e = L.blk[blockIdx.x];
-  const EnsFieldArg &E = tab[e.x];
-  const int j = (int)(((unsigned)e.y) * blockDim.x + threadIdx.x);
-  sigma_cell(E.G, j, E.f[ER], E.t_inj, E.sig, E.inject_smooth ? nullptr : E.cnt + CNT_SMAX);
 }
 
 __global__ void k_ens_smooth(const EnsFieldArg *__restrict__ tab, EnsList L, int pass) {
@@ -467,34 +741,46 @@ inline int div_up(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 }  // namespace
 
+int lossy_first_row(const pic_ctx *c) {
+  return c->d.absorb_profile != PIC_ABSORB_NONE && c->d.absorb_cells > 0
+             ? std::max(0, c->G.nr - c->G.absorb_cells - 1) : -1;
+}
+
 int ens_blocks(const pic_ctx *c, int kind) {
   const Grid &G = c->G;
-  const int gx = div_up(G.nth + 1, BX);
+  const int band = div_up(G.nth + 1, BX) * div_up(G.nr + 2 * G.g + 1, BY);  // nodes -g..nr+g, 0..nth
   switch (kind) {
-    case ENS_FLUX: return gx * div_up(G.nr + 2 * G.g + 1, BY);
-    case ENS_FILTER: return c->d.n_filt > 0 ? 3 * gx * div_up(G.nr + 2 * G.g + 1, BY) : 0;
-    case ENS_NODES: return gx * div_up(G.nr + 1, BY);
-    case ENS_LOSSY: {
-      if (c->d.absorb_profile == PIC_ABSORB_NONE || c->d.absorb_cells <= 0) return 0;
-      const int i0 = std::max(0, G.nr - G.absorb_cells - 1);
-      return gx * div_up(G.nr + 1 - i0, BY);
-    }
-    case ENS_GHOSTS: return div_up(G.nr + 1, 256);
-    case ENS_COPY32: return div_up(G.nth + 2, BX) * div_up(G.nr + 2 * G.g + 1, BY);
-    case ENS_SIGMA: return c->d.inject ? div_up(G.nth, 256) : 0;
+    case ENS_FLUX: return c->d.n_filt > FUSE_FILT ? band : 0;
+    case ENS_FILTER: return c->d.n_filt > FUSE_FILT ? 3 * band : 0;
+    case ENS_BAND: return band;
+    case ENS_SMOOTH: return c->d.inject ? div_up(G.nth, 256) : 0;
     case ENS_WRITE: return c->d.inject ? div_up((int64_t)G.nth * c->d.pairs_per_cell * 2, 256) : 0;
     default: return 0;
   }
 }
 
+// launches of the grid phases of one step (as pic_step_body makes them)
+int grid_launches(const pic_ctx *c) {
+  return (c->d.n_filt > FUSE_FILT ? 1 + 3 * c->d.n_filt : 0) + 2 + (c->d.inject ? 1 + c->d.inject_smooth : 0);
+}
+
+// whether the step's filter passes end in the scratch planes (pass by pass,
+// an odd number): F and Ft then change places
+bool filter_swaps(const pic_ctx *c) { return c->d.n_filt > FUSE_FILT && (c->d.n_filt & 1); }
+
 void ens_fill_field_arg(const pic_ctx *c, EnsFieldArg *a) {
   memset(a, 0, sizeof *a);
+  const bool fp32 = c->d.precision == PIC_FP32, fused = c->d.n_filt <= FUSE_FILT;
   a->G = c->G;
   for (int k = 0; k < 6; ++k) { a->f[k] = c->f[k]; a->f32[k] = c->f32[k]; }
   for (int k = 0; k < 3; ++k) {
-    a->Fin[k] = c->F[k];
-    a->Ftmp[k] = c->Ft[k];
-    a->Fout[k] = (c->d.n_filt & 1) ? c->Ft[k] : c->F[k];
+    a->bh[k] = c->bh[k];
+    a->epre[k] = c->epre[k];
+    // FP64: the deposit is in Ft and the filtered flux goes to F.  FP32: pass
+    // by pass the converted deposit goes to F, and Ft is the scratch.
+    a->Fin[k] = fp32 ? c->F[k] : c->Ft[k];
+    a->Ftmp[k] = fp32 ? c->Ft[k] : c->F[k];
+    a->Fout[k] = fused ? c->F[k] : ((c->d.n_filt & 1) ? a->Ftmp[k] : a->Fin[k]);
     a->acc[k] = c->acc[k];
   }
   a->grid_elems = c->grid_elems;
@@ -509,30 +795,20 @@ void ens_fill_field_arg(const pic_ctx *c, EnsFieldArg *a) {
   a->npp = c->d.pairs_per_cell;
   a->inject_smooth = c->d.inject_smooth;
   a->n_filt = c->d.n_filt;
-  a->lossy_i0 = (c->d.absorb_profile != PIC_ABSORB_NONE && c->d.absorb_cells > 0)
-                    ? std::max(0, c->G.nr - c->G.absorb_cells - 1) : -1;
+  a->lossy_i0 = lossy_first_row(c);
 }
 
 void ens_filter(const EnsFieldArg *tab, const EnsList &L, int blocks, int pass, cudaStream_t s) {
   k_ens_filter<<<(unsigned)blocks, 256, 0, s>>>(tab, L, pass);
 }
-void ens_b_half(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
-  k_ens_b_half<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
+void ens_flux(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
+  k_ens_flux<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
 }
-void ens_e_full(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
-  k_ens_e_full<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
+void ens_e_step(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
+  k_ens_e_step<<<(unsigned)blocks, dim3(BX, BY), 0, s>>>(tab, L);
 }
-void ens_lossy(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
-  k_ens_lossy<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
-}
-void ens_ghosts(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
-  k_ens_ghosts<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
-}
-void ens_copy32(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
-  k_ens_copy32<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
-}
-void ens_inject_sigma(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
-  k_ens_sigma<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
+void ens_b_step(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
+  k_ens_b_step<<<(unsigned)blocks, dim3(BX, BY), 0, s>>>(tab, L);
 }
 void ens_inject_smooth(const EnsFieldArg *tab, const EnsList &L, int blocks, int pass, cudaStream_t s) {
   k_ens_smooth<<<(unsigned)blocks, 256, 0, s>>>(tab, L, pass);
@@ -541,16 +817,43 @@ void ens_inject_write(const EnsFieldArg *tab, const EnsList &L, int blocks, cuda
   k_ens_write<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
 }
 
-void fields_b_half(pic_ctx *c) {
-  const Grid &G = c->G;
-  ++c->launches, k_b_half<<<grid2(G.nr + 1, G.nth + 1), dim3(BX, BY), 0, c->stream>>>(G, c->f[ER], c->f[ETH], c->f[EPH], c->f[BR],
-                                                                      c->f[BTH], c->f[BPH]);
+void fields_b_start(pic_ctx *c) {
+  if (c->bh_ok) return;
+  EnsFieldArg a;
+  ens_fill_field_arg(c, &a);
+  ++c->launches, k_b_start<<<grid2(c->G.nr + 1, c->G.nth + 1), dim3(BX, BY), 0, c->stream>>>(a);
+  c->bh_ok = true;
 }
 
-void fields_e_full(pic_ctx *c) {
-  const Grid &G = c->G;
-  ++c->launches, k_e_full<<<grid2(G.nr + 1, G.nth + 1), dim3(BX, BY), 0, c->stream>>>(
-      G, c->f[ER], c->f[ETH], c->f[EPH], c->f[BR], c->f[BTH], c->f[BPH], c->F[0], c->F[1], c->F[2]);
+void fields_e_step(pic_ctx *c) {
+  EnsFieldArg a;
+  ens_fill_field_arg(c, &a);
+  const bool fp32 = c->d.precision == PIC_FP32;
+  if (c->d.n_filt > FUSE_FILT) {
+    const Grid &G = c->G;
+    const dim3 gr = grid2(G.nr + 2 * G.g + 1, G.nth + 1);
+    if (fp32) ++c->launches, k_flux_from_acc<<<gr, dim3(BX, BY), 0, c->stream>>>(a);
+    for (int p = 0; p < c->d.n_filt; ++p)
+      for (int k = 0; k < 3; ++k)
+        ++c->launches, k_filter<<<gr, dim3(BX, BY), 0, c->stream>>>(G, (p & 1) ? a.Ftmp[k] : a.Fin[k],
+                                                                    (p & 1) ? a.Fin[k] : a.Ftmp[k], k == 1);
+  }
+  const unsigned nb = (unsigned)ens_blocks(c, ENS_BAND);
+  if (fp32) ++c->launches, k_e_step<true><<<nb, dim3(BX, BY), 0, c->stream>>>(a);
+  else ++c->launches, k_e_step<false><<<nb, dim3(BX, BY), 0, c->stream>>>(a);
+}
+
+void fields_b_step(pic_ctx *c, bool sigma) {
+  EnsFieldArg a;
+  ens_fill_field_arg(c, &a);
+  a.t_inj = (c->step + 1) * c->G.dt;
+  const int sg = sigma && c->d.inject ? 1 : 0;
+  const unsigned nb = (unsigned)ens_blocks(c, ENS_BAND);
+  if (c->d.precision == PIC_FP32) ++c->launches, k_b_step<true><<<nb, dim3(BX, BY), 0, c->stream>>>(a, sg);
+  else ++c->launches, k_b_step<false><<<nb, dim3(BX, BY), 0, c->stream>>>(a, sg);
+  // the filtered flux stays in F (pic_get_flux), the cleared deposit in Ft
+  if (a.Fout[0] != c->F[0])
+    for (int k = 0; k < 3; ++k) std::swap(c->F[k], c->Ft[k]);
 }
 
 void fields_copy32(pic_ctx *c) {
@@ -566,17 +869,6 @@ void fields_fill_ghosts(pic_ctx *c) {
   if (c->d.precision == PIC_FP32) fields_copy32(c);
 }
 
-void fields_finish(pic_ctx *c) {
-  const Grid &G = c->G;
-  if (c->d.absorb_profile != PIC_ABSORB_NONE && c->d.absorb_cells > 0) {
-    int i0 = G.nr - G.absorb_cells - 1;
-    if (i0 < 0) i0 = 0;
-    ++c->launches, k_lossy<<<grid2(G.nr + 1 - i0, G.nth + 1), dim3(BX, BY), 0, c->stream>>>(G, c->f[0], c->f[1], c->f[2], c->f[3],
-                                                                           c->f[4], c->f[5], i0);
-  }
-  fields_fill_ghosts(c);
-}
-
 void filter_array(pic_ctx *c, double *a, double *tmp, int half_j, int sign, int passes) {
   (void)sign;  // the fold sign is built into the weights of k_filter
   const Grid &G = c->G;
@@ -590,26 +882,16 @@ void filter_array(pic_ctx *c, double *a, double *tmp, int half_j, int sign, int 
     cudaMemcpyAsync(a, src, c->grid_elems * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
 }
 
-void fields_filter(pic_ctx *c) {
-  const int n = c->d.n_filt;
-  if (n <= 0) return;
-  const Grid &G = c->G;
-  dim3 gr = grid2(G.nr + 2 * G.g + 1, G.nth + 1);
-  for (int p = 0; p < n; ++p) {
-    for (int k = 0; k < 3; ++k)
-      ++c->launches, k_filter<<<gr, dim3(BX, BY), 0, c->stream>>>(G, c->F[k], c->Ft[k], k == 1);
-    for (int k = 0; k < 3; ++k) { double *t = c->F[k]; c->F[k] = c->Ft[k]; c->Ft[k] = t; }
-  }
-}
-
-void inject(pic_ctx *c, double t) {
+void inject(pic_ctx *c, double t, bool have_sigma) {
   const Grid &G = c->G;
   const int npp = c->d.pairs_per_cell, ns = c->d.inject_smooth;
   long long *smax = c->d_cnt + CNT_SMAX;
-  cudaMemsetAsync(smax, 0, sizeof(long long), c->stream);
   double *a = c->sig, *b = c->sig + (G.nth + 1);
   const int tb = (G.nth + 127) / 128;
-  ++c->launches, k_inject_sigma<<<tb, 128, 0, c->stream>>>(G, c->f[ER], t, a, ns ? nullptr : smax);
+  if (!have_sigma) {  // a radial slab: after the exchange of the step's fields
+    cudaMemsetAsync(smax, 0, sizeof(long long), c->stream);
+    ++c->launches, k_inject_sigma<<<tb, 128, 0, c->stream>>>(G, c->f[ER], t, a, ns ? nullptr : smax);
+  }
   for (int p = 0; p < ns; ++p) {
     ++c->launches, k_inject_smooth<<<tb, 128, 0, c->stream>>>(G.nth, a, b, p == ns - 1 ? smax : nullptr);
     double *x = a; a = b; b = x;

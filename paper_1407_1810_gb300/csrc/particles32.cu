@@ -758,61 +758,6 @@ __global__ void __launch_bounds__(NT, 4) k_ens_tiles32(const __grid_constant__ E
   tiles32_block<TI, TJ, SPEC, true>(T.A, T.P, T.maps, blockIdx.x - (unsigned)B.off[lo]);
 }
 
-// (double)v * 2^s built on the integer pipes: v rounded to 53 bits (to
-// nearest, ties to even, as the FP64 conversion does; exact for the sums
-// below 2^53 that occur in practice) and the power of two added to the
-// exponent, which is exact while the result stays normal (s in [-126, 64] here).
-// The same IEEE value as the conversion and multiply, without the FP64 pipe,
-// whose rate on this part made the conversion pass compute-bound.
-__device__ inline double fixed_to_f64(long long v, int s) {
-  if (v == 0) return 0.0;
-  const unsigned long long sign = v < 0 ? 0x8000000000000000ull : 0ull;
-  const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-  int e = 63 - __clzll((long long)m);  // m in [2^e, 2^(e+1))
-  unsigned long long mant;
-  if (e <= 52) {
-    mant = m << (52 - e);
-  } else {
-    const int sh = e - 52;
-    const unsigned long long q = m >> sh, rem = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    mant = q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull);
-    if (mant >> 53) { mant >>= 1; ++e; }
-  }
-  const unsigned long long bits = sign | ((unsigned long long)(e + s + 1023) << 52) | (mant & ((1ull << 52) - 1ull));
-  return __longlong_as_double((long long)bits);
-}
-
-// fixed point -> FP64 fluxes over the ghost band; clears the accumulators
-// (node i, j of the band -g <= i <= nr + g, 0 <= j <= nth)
-__device__ __forceinline__ void flux_node(int i, int j, int nr, int nth, int g, int PI, int LD, int PJ,
-                                          const long long *qexp, long long *a0, long long *a1, long long *a2,
-                                          double *F0, double *F1, double *F2) {
-  if (i > nr + g || j > nth) return;
-  const int s = qexp_value(qexp) - KFIX;  // one flux unit is 2^s of charge
-  const size_t o = (size_t)(i + PI) * LD + (size_t)(j + PJ);
-  F0[o] = fixed_to_f64(a0[o], s); a0[o] = 0;
-  F1[o] = fixed_to_f64(a1[o], s); a1[o] = 0;
-  F2[o] = fixed_to_f64(a2[o], s); a2[o] = 0;
-}
-
-__global__ void k_flux_from_acc(int nr, int nth, int g, int PI, int PJ, int LD, const long long *qexp,
-                                long long *a0, long long *a1, long long *a2, double *F0, double *F1, double *F2) {
-  flux_node(-g + (int)(blockIdx.y * 8 + threadIdx.y), blockIdx.x * 32 + threadIdx.x, nr, nth, g, PI, LD, PJ, qexp,
-            a0, a1, a2, F0, F1, F2);
-}
-
-// the same over the members of an ensemble: 256-thread blocks, each member's
-// band covered by 32 x 8 node blocks as above
-__global__ void k_ens_flux(const EnsFieldArg *__restrict__ tab, EnsList L) {
-  const int2 e = L.blk[blockIdx.x];
-  const EnsFieldArg &E = tab[e.x];
-  const Grid &G = E.G;
-  const unsigned b = (unsigned)e.y, gx = (unsigned)(G.nth + 1 + 31) / 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  flux_node(-G.g + (int)((b / gx) * 8 + ty), (int)((b % gx) * 32 + tx), G.nr, G.nth, G.g, G.PI, G.LD, G.PJ,
-            E.qexp, E.acc[0], E.acc[1], E.acc[2], E.Fin[0], E.Fin[1], E.Fin[2]);
-}
-
 // ---- counting sort into tile bins (drops removed particles) ---------------
 // Bins are numbered cell by cell, tile-major: key = tile * tc + cell index
 // inside the tile; removed particles go to the last bin, ntiles * tc.  Keys
@@ -1306,23 +1251,22 @@ int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaSt
   return launches;
 }
 
-void ens_flux_from_acc(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s) {
-  k_ens_flux<<<(unsigned)blocks, 256, 0, s>>>(tab, L);
+// Particles per work unit.  A context on its own: no more than about 1216
+// units besides one per tile (two waves of 4 CTAs on each of the 152 SMs), so
+// a large run keeps one unit per tile while the tiles of a small plasma are
+// spread over the chip; and at least two passes of a CTA's threads, below
+// which a CTA's window and flush cost more than its particles.  (72 x 56
+// rotator, 1e5 particles, 20 steps with the fields read out: 0.91 ms with
+// units of 512, 0.96 with 1024, 1.10 with 2048, 1.39 with 4096.)  Members of
+// an ensemble share the chip: their units follow the particles of all of them
+// (64 members, 2.4e7 particles: 62 ms for 40 steps with units of 4096, 64 with
+// 2048, 71 with 1024, 78 with 512).
+constexpr int64_t UNIT_MIN = 2 * NT, UNITS_ALONE = 2 * 4 * 152, UNITS_ENSEMBLE = 8 * 4 * 152;
+static int64_t unit_size(const pic_ctx *c) {
+  const int64_t n = c->ens_particles > 0 ? c->ens_particles : c->n_used;
+  const int64_t units = c->ens_particles > 0 ? UNITS_ENSEMBLE : UNITS_ALONE;
+  return std::max(UNIT_MIN, ((n + units - 1) / units + NT - 1) / NT * NT);
 }
-
-void flux_from_acc(pic_ctx *c) {
-  const Grid &G = c->G;
-  dim3 gr((G.nth + 1 + 31) / 32, (G.nr + 2 * G.g + 1 + 7) / 8);
-  ++c->launches, k_flux_from_acc<<<gr, dim3(32, 8), 0, c->stream>>>(G.nr, G.nth, G.g, G.PI, G.PJ, G.LD, c->qexp,
-                                                     c->acc[0], c->acc[1], c->acc[2], c->F[0], c->F[1], c->F[2]);
-}
-
-// Particles per work unit: at least UNIT_MIN, and large enough that a run
-// holds no more than about UNIT_TARGET units besides one per tile (two waves of
-// 4 CTAs on each of the 152 SMs): a large run keeps one unit per tile, while
-// the dense tiles of a small plasma are spread over many CTAs instead of
-// holding the whole kernel back on one.
-constexpr int64_t UNIT_MIN = 4096, UNIT_TARGET = 2 * 4 * 152;
 
 int64_t sort32(pic_ctx *c) {
   Tiles &T = c->tiles;
@@ -1336,7 +1280,7 @@ int64_t sort32(pic_ctx *c) {
   // room for the work units first: on failure no particle has moved, every
   // particle takes the unbinned path until a sort succeeds, and the context
   // reports the error
-  T.unit = std::max(UNIT_MIN, (n + UNIT_TARGET - 1) / UNIT_TARGET);
+  T.unit = unit_size(c);
   const int64_t ucap = T.ntiles + n / T.unit + 1;
   if (ucap > T.units_cap) {
     cudaStreamSynchronize(c->stream);
@@ -1410,7 +1354,7 @@ int ens_sort32(pic_ctx *const *cs, int m, cudaStream_t st, EnsSortScratch &sc, i
   bool synced = false;
   for (pic_ctx *c : due) {
     Tiles &T = c->tiles;
-    T.unit = std::max(UNIT_MIN, (c->n_used + UNIT_TARGET - 1) / UNIT_TARGET);
+    T.unit = unit_size(c);
     const int64_t ucap = T.ntiles + c->n_used / T.unit + 1;
     if (ucap <= T.units_cap) continue;
     if (!synced) { PIC_CUDA(cudaStreamSynchronize(st)); synced = true; }

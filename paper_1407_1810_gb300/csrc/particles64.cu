@@ -238,7 +238,7 @@ void particles64(pic_ctx *c, double t) {
   if (c->n_used == 0) return;
   Fields64 F;
   for (int k = 0; k < 6; ++k) F.f[k] = c->f[k];
-  Flux64 D{c->F[0], c->F[1], c->F[2]};
+  Flux64 D{c->Ft[0], c->Ft[1], c->Ft[2]};  // the deposit planes, cleared by the last step
   const int64_t blocks = (c->n_used + 255) / 256;
   ++c->launches, k_particles64<<<(unsigned)blocks, 256, 0, c->stream>>>(c->G, c->p64, c->n_used, t, F, D, c->d_err, c->d_cnt,
                                                                           axis_ties(c));

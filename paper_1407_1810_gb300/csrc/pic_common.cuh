@@ -54,11 +54,10 @@ struct Metric {
   const double *bT0, *bT1;          // h 2 r_i / (r_{i+1}^2 - r_i^2), same with r_{i+1}  (B_th, B_ph)
   const double *bP;                 // h 2 (r_{i+1} - r_i) / (r_{i+1}^2 - r_i^2)  (B_ph)
   const double *eR;                 // dt / rb_i                                (E_r)
-  const double *eT0, *eT1;          // dt 2 rb_{i-1} / (rb_i^2 - rb_{i-1}^2), same with rb_i  (E_th, E_ph)
-  const double *eP;                 // dt 2 (rb_i - rb_{i-1}) / (rb_i^2 - rb_{i-1}^2)  (E_ph)
   const double *cB1, *cB2;          // sin th_j / dcos_j, sin th_{j+1} / dcos_j  (B_r)
   const double *cE1, *cE2;          // sin tb_j / dcos_tb_j, sin tb_{j-1} / dcos_tb_j  (E_r)
   const double *cF;                 // 1 / (2 pi sin tb_j)                      (E_th flux)
+  const double *w0, *w1, *wd;       // dt rb_{i-1}, dt rb_i, dt (rb_i - rb_{i-1})  (E_th, E_ph)
 };
 
 struct Grid {
@@ -84,6 +83,60 @@ __host__ __device__ inline size_t gidx(const Grid &G, int i, int j) {
 }
 
 constexpr double PI_D = 3.14159265358979323846;
+
+// (double)v * 2^s built on the integer pipes: v rounded to 53 bits (to
+// nearest, ties to even, as the FP64 conversion does; exact for the sums
+// below 2^53 that occur in practice) and the power of two added to the
+// exponent, which is exact while the result stays normal (s in [-126, 64] here).
+// The same IEEE value as the conversion and multiply, without the FP64 pipe,
+// whose rate on this part made the conversion pass compute-bound.
+__device__ inline double fixed_to_f64(long long v, int s) {
+  if (v == 0) return 0.0;
+  const unsigned long long sign = v < 0 ? 0x8000000000000000ull : 0ull;
+  const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  int e = 63 - __clzll((long long)m);  // m in [2^e, 2^(e+1))
+  unsigned long long mant;
+  if (e <= 52) {
+    mant = m << (52 - e);
+  } else {
+    const int sh = e - 52;
+    const unsigned long long q = m >> sh, rem = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
+    mant = q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull);
+    if (mant >> 53) { mant >>= 1; ++e; }
+  }
+  const unsigned long long bits = sign | ((unsigned long long)(e + s + 1023) << 52) | (mant & ((1ull << 52) - 1ull));
+  return __longlong_as_double((long long)bits);
+}
+
+// the same for a 128-bit sum (flux sums that leave no room for the filter's
+// weights in 64 bits)
+__device__ inline double fixed_to_f64(__int128 v, int s) {
+  const bool neg = v < 0;
+  const unsigned __int128 m = neg ? (unsigned __int128)0 - (unsigned __int128)v : (unsigned __int128)v;
+  const unsigned long long hi = (unsigned long long)(m >> 64);
+  if (hi == 0 && !(unsigned long long)(m >> 63)) return fixed_to_f64((long long)v, s);
+  // keep the top 62 or 63 bits; the rest only decides ties (sticky bit)
+  const int sh = hi ? 66 - __clzll((long long)hi) : 2;
+  unsigned long long t = (unsigned long long)(m >> sh);
+  if (m & ((((unsigned __int128)1) << sh) - 1)) t |= 1ull;
+  const long long r = (long long)t;
+  return fixed_to_f64(neg ? -r : r, s + sh);
+}
+
+// (float)x rounded to nearest even, on the integer pipes: the conversion
+// instruction runs on the FP64 pipe, 64 issue slots a warp on this part
+__device__ inline float f64_to_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u < 254u) {  // a normal FP32 result (or one rounded up to infinity)
+    unsigned r = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned rem = lo & 0x1fffffffu;
+    r += (rem > 0x10000000u || (rem == 0x10000000u && (r & 1u))) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | r);
+  }
+  if (e == 0) return __uint_as_float(hi & 0x80000000u);
+  return (float)x;  // subnormal results, overflow, infinities and NaN
+}
 
 // ---- stretching functions, Sec. 3.2 -----------------------------------------
 __device__ inline double map_r(const Grid &G, double x1) {

@@ -102,13 +102,15 @@ struct EnsList {
 enum ProfSlot { PROF_PARTICLES = 0, PROF_REDUCE = 1, PROF_FILTER = 2, PROF_FIELDS = 3, PROF_INJECT = 4,
                 PROF_SORT = 5, PROF_N };
 
-// One FP32 member at one step as the batched grid kernels read it: the
-// member's grid and arrays, the flux buffers as the step starts, after its
-// filter passes and their scratch, and the step's injection.
+// One context at one step as the grid kernels read it (kernel parameter of a
+// single context's launches, device table of an ensemble's): its grid and
+// arrays, the flux buffers and the step's injection.
 struct EnsFieldArg {
   Grid G;
   double *f[6];
-  double *Fin[3], *Ftmp[3], *Fout[3];  // flux written by the deposit; filter scratch; flux the E update reads
+  double *bh[3];                       // B at the half step (see fields.cu)
+  double *epre[3];                     // E of rows lossy_i0..nr before the lossy layer
+  double *Fin[3], *Ftmp[3], *Fout[3];  // FP64 deposit; scratch of the pass-by-pass filter; filtered flux
   float *f32[6];
   long long *acc[3];
   size_t grid_elems;
@@ -125,8 +127,7 @@ struct EnsFieldArg {
 };
 
 // kinds of batched grid launch (block counts per member: ens_blocks)
-enum EnsKind { ENS_FLUX = 0, ENS_FILTER, ENS_NODES, ENS_LOSSY, ENS_GHOSTS, ENS_COPY32, ENS_SIGMA, ENS_WRITE,
-               ENS_NKIND };
+enum EnsKind { ENS_FLUX = 0, ENS_FILTER, ENS_BAND, ENS_SMOOTH, ENS_WRITE, ENS_NKIND };
 
 }  // namespace pic
 
@@ -138,8 +139,11 @@ struct pic_ctx {
   double *metric_buf = nullptr;
   size_t grid_elems = 0;  // elements of one padded grid array
   double *f[6] = {};      // plasma fields (FP64)
+  double *bh[3] = {};     // B half a step ahead: B + (dt/2) curl E of the stored fields
+  bool bh_ok = false;     // bh matches the stored fields (fields_b_start)
+  double *epre[3] = {};   // E of the lossy rows before the layer acts, between the E and B updates
   double *F[3] = {};      // fluxes of the current step (FP64, after filtering)
-  double *Ft[3] = {};     // filter double buffer
+  double *Ft[3] = {};     // FP64 path: the deposit; FP32 path: scratch of a pass-by-pass filter
   float *f32[6] = {};     // FP32 gather copies (FP32 path)
   float *r_n32 = nullptr; // f_r(i) per padded row, FP32 (FP32 path)
   float2 *th_n32 = nullptr; // (sin, cos) of the linear map's node angle per padded column (FP32 path)
@@ -174,6 +178,7 @@ struct pic_ctx {
   int host_err = 0;
   int steps_since_sort = 0;
   bool need_sort = false;
+  int64_t ens_particles = 0;  // particles of all members while an ensemble advances this context, else 0
   bool small_steps = false; // FP32: the grid bounds the move's series arguments (series without fallback)
   bool mix_sort = true;    // FP32: the next sort orders by cell and mixes each tile's bin
   // profiling: one start/stop event pair per phase per step, read back lazily
@@ -188,13 +193,15 @@ struct pic_ctx {
 
 namespace pic {
 // fields.cu
-void fields_b_half(pic_ctx *c);
-void fields_e_full(pic_ctx *c);
-void fields_finish(pic_ctx *c);        // lossy layer + axis ghosts (+ FP32 copies)
-void fields_filter(pic_ctx *c);        // n_filt passes on F
+int lossy_first_row(const pic_ctx *c);  // -1: no lossy layer
+void fields_b_start(pic_ctx *c);       // bh of the stored fields, when it does not match them
+void fields_e_step(pic_ctx *c);        // filtered flux of the deposit, E update, lossy layer on E
+void fields_b_step(pic_ctx *c, bool sigma);  // B update, lossy layer, ghosts, FP32 copies; clears the deposit;
+                                             // sigma: the injection's surface charge at the step's end
 void fields_fill_ghosts(pic_ctx *c);   // axis ghosts (+ FP32 copies) (after pic_set_fields)
 void fields_copy32(pic_ctx *c);        // FP32 gather copies of the fields (FP32 path)
-void inject(pic_ctx *c, double t);     // surface pairs into slots [n_used, n_used + 2 npp nth)
+// surface pairs into slots [n_used, n_used + 2 npp nth); have_sigma: fields_b_step formed the surface charge
+void inject(pic_ctx *c, double t, bool have_sigma);
 void moments(pic_ctx *c, bool snapshot, pic_moments *out);
 void luminosity(pic_ctx *c, double t, double *L);  // nr + 1 device values (Sec. 5.3)
 void filter_array(pic_ctx *c, double *a, double *tmp, int half_j, int sign, int passes);
@@ -211,12 +218,11 @@ void reduce_particles64(pic_ctx *c);   // kinetic energy, live count, total char
 int ens_blocks(const pic_ctx *c, int kind);  // blocks one member needs in a launch of that kind
 void ens_fill_field_arg(const pic_ctx *c, EnsFieldArg *a);  // the member's arrays (not the step's values)
 void ens_filter(const EnsFieldArg *tab, const EnsList &L, int blocks, int pass, cudaStream_t s);
-void ens_b_half(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
-void ens_e_full(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
-void ens_lossy(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
-void ens_ghosts(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
-void ens_copy32(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
-void ens_inject_sigma(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
+void ens_flux(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
+void ens_e_step(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
+void ens_b_step(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
+int grid_launches(const pic_ctx *c);
+bool filter_swaps(const pic_ctx *c);
 void ens_inject_smooth(const EnsFieldArg *tab, const EnsList &L, int blocks, int pass, cudaStream_t s);
 void ens_inject_write(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
 // particles32.cu
@@ -231,7 +237,6 @@ void ens_tile_arg(pic_ctx *c, double t, void *out);  // the member's tile-kernel
 // arguments, ens_tile_arg_bytes() each, and their block counts); returns the
 // number of kernels launched (members are taken in groups of up to 48)
 int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaStream_t s);
-void ens_flux_from_acc(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
 // the tile sort of m FP32 contexts at once on stream st (each launch serves
 // every member; one read-back, one synchronisation); the staging buffers
 // persist in sc between calls.  *kernels: the kernels launched.
@@ -242,7 +247,6 @@ struct EnsSortScratch {
 int ens_sort32(pic_ctx *const *cs, int m, cudaStream_t st, EnsSortScratch &sc, int64_t *kernels);
 void ens_sort_scratch_free(EnsSortScratch &sc);
 void particles32(pic_ctx *c, double t);
-void flux_from_acc(pic_ctx *c);        // fixed point -> FP64 fluxes, clears the accumulators
 int64_t sort32(pic_ctx *c);            // tile sort + removal; returns live count
 void charge32(pic_ctx *c, double *Q, double *Qa);
 void reduce_particles32(pic_ctx *c);

@@ -2,7 +2,7 @@
 // the paper runs over MPI, Sec. 2), each slab a context of its own, with the
 // exchanges a step needs between neighbouring slabs:
 //
-//   * field halo: after each Yee sub-step, the rows next to an interface are
+//   * field halo: after the E and the B update, the rows next to an interface are
 //     copied to the neighbour's ghost rows (the gather reads one ghost row on
 //     each side, the curl one row of E or B across the interface);
 //   * flux halo: the charge a slab's particles deposit into rows owned by the
@@ -383,31 +383,25 @@ int slab_step(pic_slabs *g) {
   const double t = g->step * g->d.dt;
   int e;
   if (g->d.precision == PIC_FP32) {
-    // exact int64 sums across the interfaces, then the conversion
+    // exact int64 sums across the interfaces, before the filter
     for (pic_ctx *c : g->ctx) particles32(c, t);
     for (int s = 0; s + 1 < S; ++s)
       for (int k = 0; k < 3; ++k)
         if ((e = halo_sum(g, g->ctx[s], g->ctx[s + 1], g->ctx[s]->acc[k], g->ctx[s + 1]->acc[k]))) return e;
-    for (pic_ctx *c : g->ctx) flux_from_acc(c);
   } else {
-    for (pic_ctx *c : g->ctx) {
-      for (int k = 0; k < 3; ++k) cudaMemsetAsync(c->F[k], 0, c->grid_elems * sizeof(double), g->stream);
-      particles64(c, t);
-    }
+    for (pic_ctx *c : g->ctx) particles64(c, t);
     for (int s = 0; s + 1 < S; ++s)
       for (int k = 0; k < 3; ++k)
-        if ((e = halo_sum(g, g->ctx[s], g->ctx[s + 1], g->ctx[s]->F[k], g->ctx[s + 1]->F[k]))) return e;
+        if ((e = halo_sum(g, g->ctx[s], g->ctx[s + 1], g->ctx[s]->Ft[k], g->ctx[s + 1]->Ft[k]))) return e;
   }
-  if (g->d.n_filt > 0)
-    for (pic_ctx *c : g->ctx) fields_filter(c);
-  static const int B3[3] = {BR, BTH, BPH}, E3[3] = {ER, ETH, EPH}, ALL[6] = {ER, ETH, EPH, BR, BTH, BPH};
-  for (pic_ctx *c : g->ctx) fields_b_half(c);
-  if ((e = exchange_fields(g, B3, 3))) return e;
-  for (pic_ctx *c : g->ctx) fields_e_full(c);
+  static const int B3[3] = {BR, BTH, BPH}, E3[3] = {ER, ETH, EPH};
+  for (pic_ctx *c : g->ctx) fields_e_step(c);
   if ((e = exchange_fields(g, E3, 3))) return e;
-  for (pic_ctx *c : g->ctx) fields_b_half(c);
-  for (pic_ctx *c : g->ctx) fields_finish(c);
-  if ((e = exchange_fields(g, ALL, 6))) return e;
+  for (pic_ctx *c : g->ctx) fields_b_step(c, false);
+  if ((e = exchange_fields(g, E3, 3)) || (e = exchange_fields(g, B3, 3))) return e;  // with the axis ghosts
+  for (int s = 0; s + 1 < S; ++s)
+    for (int k = 0; k < 3; ++k)
+      if ((e = halo_set(g, g->ctx[s], g->ctx[s + 1], g->ctx[s]->bh[k], g->ctx[s + 1]->bh[k], 2))) return e;
   if (g->d.precision == PIC_FP32)  // the gather copies again, now with the neighbours' rows
     for (pic_ctx *c : g->ctx) fields_copy32(c);
   g->step += 1;
@@ -417,7 +411,7 @@ int slab_step(pic_slabs *g) {
     const int64_t slots = (int64_t)2 * g->d.pairs_per_cell * g->d.nth;
     if ((e = room(c0, slots))) return e;
     c0->next_id = g->next_id;
-    inject(c0, g->step * g->d.dt);
+    inject(c0, g->step * g->d.dt, false);
     g->next_id = c0->next_id;
   }
   if ((e = migrate(g))) return e;
