@@ -546,6 +546,19 @@ int pic_create_context(pic_ctx **out, const pic_desc &d, void *stream, int i0, i
   }
   cudaMemset(c->Q, 0, ge * 8); cudaMemset(c->Qa, 0, ge * 8); cudaMemset(c->Qt, 0, ge * 8);
   cudaMemset(c->gsnap, 0, ge * 8);
+  // sine and cosine of the node angle pi j / nth of the linear theta map at
+  // padded column jj, each the sine of an angle measured from the nearer pole
+  // or from the equator (exact zeros and ones at the poles and the equator)
+  auto node_angle = [&](int jj) {
+    const double j = (double)(jj - G.PJ), m = std::min(j, d.nth - j);
+    return make_double2(std::sin(M_PI * m / d.nth), std::sin(M_PI * (d.nth - 2.0 * j) / (2.0 * d.nth)));
+  };
+  if (d.precision == PIC_FP64) {
+    std::vector<double2> tn(G.LD);
+    for (int jj = 0; jj < G.LD; ++jj) tn[jj] = node_angle(jj);
+    if ((e = dalloc(&c->th_n64, tn.size()))) return fail(e);
+    PIC_CUDA(cudaMemcpy(c->th_n64, tn.data(), tn.size() * sizeof(double2), cudaMemcpyHostToDevice));
+  }
   if (d.precision == PIC_FP32) {
     for (int k = 0; k < 6; ++k) {
       if ((e = dalloc(&c->f32[k], ge))) return fail(e);
@@ -570,14 +583,10 @@ int pic_create_context(pic_ctx **out, const pic_desc &d, void *stream, int i0, i
       c->small_steps = d.r_map == PIC_R_LOG && G.dxi <= 1.0 / 16 && G.dt / h_fr(d, G.dxi, -G.g) <= 1.0 / 40;
       if ((e = dalloc(&c->r_n32, rn.size()))) return fail(e);
       PIC_CUDA(cudaMemcpy(c->r_n32, rn.data(), rn.size() * sizeof(float), cudaMemcpyHostToDevice));
-      // sine and cosine of the node angle pi j / nth of the linear theta map
-      // per padded column, each the sine of an angle measured from the nearer
-      // pole or from the equator (exact zeros and ones at the poles and the
-      // equator), rounded once to FP32
       std::vector<float2> tn(G.LD);
       for (int jj = 0; jj < G.LD; ++jj) {
-        const double j = (double)(jj - G.PJ), m = std::min(j, d.nth - j);
-        tn[jj] = make_float2((float)std::sin(M_PI * m / d.nth), (float)std::sin(M_PI * (d.nth - 2.0 * j) / (2.0 * d.nth)));
+        const double2 a = node_angle(jj);
+        tn[jj] = make_float2((float)a.x, (float)a.y);
       }
       if ((e = dalloc(&c->th_n32, tn.size()))) return fail(e);
       PIC_CUDA(cudaMemcpy(c->th_n32, tn.data(), tn.size() * sizeof(float2), cudaMemcpyHostToDevice));
@@ -1101,6 +1110,7 @@ extern "C" int pic_destroy(pic_ctx *c) {
   for (int k = 0; k < 6; ++k) { cudaFree(c->f[k]); cudaFree(c->f32[k]); }
   cudaFree(c->r_n32);
   cudaFree(c->th_n32);
+  cudaFree(c->th_n64);
   cudaFree(c->d_tile_maps);
   for (int k = 0; k < 3; ++k) { cudaFree(c->F[k]); cudaFree(c->Ft[k]); cudaFree(c->acc[k]); cudaFree(c->bh[k]); cudaFree(c->epre[k]); }
   cudaFree(c->Q); cudaFree(c->Qa); cudaFree(c->Qt); cudaFree(c->gsnap); cudaFree(c->sig);

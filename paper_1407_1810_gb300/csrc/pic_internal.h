@@ -147,6 +147,7 @@ struct pic_ctx {
   float *f32[6] = {};     // FP32 gather copies (FP32 path)
   float *r_n32 = nullptr; // f_r(i) per padded row, FP32 (FP32 path)
   float2 *th_n32 = nullptr; // (sin, cos) of the linear map's node angle per padded column (FP32 path)
+  double2 *th_n64 = nullptr; // the same in FP64 (FP64 path)
   long long *acc[3] = {}; // fixed-point flux accumulators (FP32 path)
   alignas(64) unsigned char tile_maps[3][6 * 128] = {}; // FP32: field tensor maps per tile shape (TMA)
   unsigned char *d_tile_maps = nullptr;  // the same maps in device memory (batched ensemble launches)
