@@ -838,11 +838,9 @@ extern "C" int pic_get_charge(pic_ctx *c, int32_t filtered, double *out, int64_t
   const size_t plane = (size_t)rows * cols;
   *n = (int64_t)plane;
   if (!out) return PIC_OK;
-  cudaMemsetAsync(c->Q, 0, c->grid_elems * sizeof(double), c->stream);
-  cudaMemsetAsync(c->Qa, 0, c->grid_elems * sizeof(double), c->stream);
-  if (c->d.precision == PIC_FP32) charge32(c, c->Q, c->Qa);
-  else charge64(c, c->Q, c->Qa);
-  if (filtered) filter_array(c, c->Q, c->Qt, 0, +1, c->d.n_filt);
+  if (c->d.precision == PIC_FP32) charge32(c);
+  else charge64(c);
+  if (filtered) filter_charge(c);
   double *tmp;
   PIC_CUDA(cudaMalloc((void **)&tmp, plane * sizeof(double)));
   dim3 gr((cols + 31) / 32, (rows + 7) / 8);

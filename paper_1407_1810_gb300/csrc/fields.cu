@@ -282,6 +282,25 @@ __constant__ int FILT_W[FUSE_FILT + 1][FUSE_FILT + 1] = {  // C(2N, N + k)
 // Images of a tile's rows and columns, formed once per block: array offset (or
 // -1: zero) and factor (+-1, +-2) of row i0 - N + r and, for integer and
 // half-integer j, of column j0 - N + q of the continued deposit.
+//
+// FP64 tiles take the weights from a table of doubles and the factors through
+// the exponent and sign bits: an integer-to-double conversion or a product
+// costs as much of the FP64 pipe as an addition of the convolution.
+__constant__ double FILT_WD[FUSE_FILT + 1][FUSE_FILT + 1] = {
+    {1, 0, 0, 0, 0}, {2, 1, 0, 0, 0}, {6, 4, 1, 0, 0}, {20, 15, 6, 1, 0}, {70, 56, 28, 8, 1}};
+template <class T>
+__device__ __forceinline__ T filt_weight(int N, int k) { return T(FILT_W[N][k]); }
+template <>
+__device__ __forceinline__ double filt_weight<double>(int N, int k) { return FILT_WD[N][k]; }
+template <class T>
+__device__ __forceinline__ T filt_scaled(int c, T v) { return T(c) * v; }
+template <>
+__device__ __forceinline__ double filt_scaled<double>(int c, double v) {
+  int hi = __double2hiint(v);
+  if ((c == 2 || c == -2) && (hi & 0x7ff00000) != 0) hi += 0x00100000;  // doubled (zeros stay)
+  return __hiloint2double(c < 0 ? hi ^ 0x80000000 : hi, __double2loint(v));
+}
+
 struct FiltImages {
   int row[TH], col[2][TW];
   signed char row_c[TH], col_c[2][TW];
@@ -336,8 +355,8 @@ __device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &
         if (r < h && q < w) {
           const int ro = im.row[r];
           t.in[k][r][q] = ro < 0 ? T(0)
-                                 : T(im.row_c[r] * im.col_c[half][q]) *
-                                       load(c0 + k, (size_t)ro * G.LD + im.col[half][q]);
+                                 : filt_scaled<T>(im.row_c[r] * im.col_c[half][q],
+                                                  load(c0 + k, (size_t)ro * G.LD + im.col[half][q]));
         }
       }
   __syncthreads();
@@ -348,16 +367,16 @@ __device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &
 #pragma unroll
       for (int k = 0; k < NC; ++k) {
         const T *x = &t.in[k][r][tx + N];
-        T s = T(FILT_W[N][0]) * x[0];
-        for (int m = 1; m <= N; ++m) s += T(FILT_W[N][m]) * (x[-m] + x[m]);
+        T s = filt_weight<T>(N, 0) * x[0];
+        for (int m = 1; m <= N; ++m) s += filt_weight<T>(N, m) * (x[-m] + x[m]);
         t.mid[k][r][tx] = s;
       }
   }
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
-    T s = T(FILT_W[N][0]) * t.mid[k][ty + N][tx];
-    for (int m = 1; m <= N; ++m) s += T(FILT_W[N][m]) * (t.mid[k][ty + N - m][tx] + t.mid[k][ty + N + m][tx]);
+    T s = filt_weight<T>(N, 0) * t.mid[k][ty + N][tx];
+    for (int m = 1; m <= N; ++m) s += filt_weight<T>(N, m) * (t.mid[k][ty + N - m][tx] + t.mid[k][ty + N + m][tx]);
     out[k] = s;
   }
 }
@@ -454,6 +473,21 @@ __device__ __forceinline__ void b_block(const EnsFieldArg &S, unsigned b, bool s
   if (i < 0 || i > G.nr) return;
   b_node<FP32>(S, i, j);
   if (sigma && i == 0) sigma_cell(G, j, S.f[ER], S.t_inj, S.sig, S.inject_smooth ? nullptr : S.cnt + CNT_SMAX);
+}
+
+// the passes of an integer-j FP64 array (the node charge) in one
+__global__ void __launch_bounds__(BX *BY) k_filter_tile(Grid G, const double *__restrict__ a, double *__restrict__ out,
+                                                       int N) {
+  __shared__ FiltImages im;
+  __shared__ FiltTile<double, 1> t;
+  const int i0 = -G.g + (int)blockIdx.y * BY, j0 = (int)blockIdx.x * BX;
+  double v[1];
+  filt_images(im, G, i0, j0, N);
+  filt_conv(t, im, G, N, 0, v, [&](int, size_t x) { return a[x]; });
+  const int i = i0 + (int)threadIdx.y, j = j0 + (int)threadIdx.x;
+  if (i > G.nr + G.g || j > G.nth) return;
+  const double sc = __longlong_as_double((long long)(1023 - 4 * N) << 52);  // 16^-N
+  out[gidx(G, i, j)] = v[0] * (j == 0 || j == G.nth ? 0.5 * sc : sc);
 }
 
 template <bool FP32>
@@ -869,17 +903,19 @@ void fields_fill_ghosts(pic_ctx *c) {
   if (c->d.precision == PIC_FP32) fields_copy32(c);
 }
 
-void filter_array(pic_ctx *c, double *a, double *tmp, int half_j, int sign, int passes) {
-  (void)sign;  // the fold sign is built into the weights of k_filter
+void filter_charge(pic_ctx *c) {
   const Grid &G = c->G;
-  dim3 gr = grid2(G.nr + 2 * G.g + 1, G.nth + 1);
-  double *src = a, *dst = tmp;
-  for (int p = 0; p < passes; ++p) {
-    ++c->launches, k_filter<<<gr, dim3(BX, BY), 0, c->stream>>>(G, src, dst, half_j);
-    double *t = src; src = dst; dst = t;
+  const int n = c->d.n_filt;
+  const dim3 gr = grid2(G.nr + 2 * G.g + 1, G.nth + 1);
+  if (n == 0) return;
+  if (n <= FUSE_FILT) {
+    ++c->launches, k_filter_tile<<<gr, dim3(BX, BY), 0, c->stream>>>(G, c->Q, c->Qt, n);
+    std::swap(c->Q, c->Qt);
   }
-  if (src != a)
-    cudaMemcpyAsync(a, src, c->grid_elems * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
+  for (int p = 0; n > FUSE_FILT && p < n; ++p) {
+    ++c->launches, k_filter<<<gr, dim3(BX, BY), 0, c->stream>>>(G, c->Q, c->Qt, 0);
+    std::swap(c->Q, c->Qt);
+  }
 }
 
 void inject(pic_ctx *c, double t, bool have_sigma) {
@@ -968,11 +1004,9 @@ void field_energy_rows(pic_ctx *c, int imax) {
 
 void moments(pic_ctx *c, bool snapshot, pic_moments *out) {
   const Grid &G = c->G;
-  cudaMemsetAsync(c->Q, 0, c->grid_elems * sizeof(double), c->stream);
-  cudaMemsetAsync(c->Qa, 0, c->grid_elems * sizeof(double), c->stream);
-  if (c->d.precision == PIC_FP32) charge32(c, c->Q, c->Qa);
-  else charge64(c, c->Q, c->Qa);
-  filter_array(c, c->Q, c->Qt, 0, +1, c->d.n_filt);
+  if (c->d.precision == PIC_FP32) charge32(c);
+  else charge64(c);
+  filter_charge(c);
   int L = c->d.absorb_profile == PIC_ABSORB_NONE ? 0 : c->d.absorb_cells;
   int imax = G.nr - L - 1;
   cudaMemsetAsync(c->d_cnt + CNT_GMAX, 0, 2 * sizeof(long long), c->stream);

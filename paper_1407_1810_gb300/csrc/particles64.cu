@@ -518,10 +518,11 @@ int64_t compact64(pic_ctx *c) {
   return live;
 }
 
-void charge64(pic_ctx *c, double *Q, double *Qa) {
+void charge64(pic_ctx *c) {
+  for (double *p : {c->Q, c->Qa}) cudaMemsetAsync(p, 0, c->grid_elems * sizeof(double), c->stream);
   if (c->n_used == 0) return;
   ++c->launches, k_charge64<<<(unsigned)((c->n_used + 255) / 256), 256, 0, c->stream>>>(c->G, c->p64.x1, c->p64.x2, c->p64.qw,
-                                                                        c->n_used, Q, Qa);
+                                                                        c->n_used, c->Q, c->Qa);
 }
 
 void reduce_particles64(pic_ctx *c) {

@@ -205,7 +205,7 @@ void fields_copy32(pic_ctx *c);        // FP32 gather copies of the fields (FP32
 void inject(pic_ctx *c, double t, bool have_sigma);
 void moments(pic_ctx *c, bool snapshot, pic_moments *out);
 void luminosity(pic_ctx *c, double t, double *L);  // nr + 1 device values (Sec. 5.3)
-void filter_array(pic_ctx *c, double *a, double *tmp, int half_j, int sign, int passes);
+void filter_charge(pic_ctx *c);        // the current's filter on Q (Qt is scratch)
 // Gauss law (G - Qbar against the snapshot, into d_cnt[CNT_GMAX/QMAX]) over
 // local rows ilo..imax, with Q, Qa already deposited and filtered
 void gauss_rows(pic_ctx *c, int ilo, int imax, bool snapshot);
@@ -213,7 +213,7 @@ void field_energy_rows(pic_ctx *c, int imax);  // adds rows 0..imax to d_acc[ACC
 // particles64.cu
 void particles64(pic_ctx *c, double t);
 int64_t compact64(pic_ctx *c);         // stable removal of dead slots; returns live count
-void charge64(pic_ctx *c, double *Q, double *Qa);
+void charge64(pic_ctx *c);             // the same, FP64 path
 void reduce_particles64(pic_ctx *c);   // kinetic energy, live count, total charge
 // batched launches over ensemble members (fields.cu); blocks: the launch's grid
 int ens_blocks(const pic_ctx *c, int kind);  // blocks one member needs in a launch of that kind
@@ -249,7 +249,7 @@ int ens_sort32(pic_ctx *const *cs, int m, cudaStream_t st, EnsSortScratch &sc, i
 void ens_sort_scratch_free(EnsSortScratch &sc);
 void particles32(pic_ctx *c, double t);
 int64_t sort32(pic_ctx *c);            // tile sort + removal; returns live count
-void charge32(pic_ctx *c, double *Q, double *Qa);
+void charge32(pic_ctx *c);             // node charge Q and sum |qw| Qa (Qt is scratch)
 void reduce_particles32(pic_ctx *c);
 // the tie log and hints of a context for the step it is taking
 inline AxisTies axis_ties(const pic_ctx *c);

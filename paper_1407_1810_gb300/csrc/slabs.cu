@@ -343,10 +343,8 @@ int migrate(pic_slabs *g) {
 // interior rows (nodes 1 <= i <= nr - absorb_cells - 1 of the whole grid)
 int slab_gauss(pic_slabs *g, bool snapshot, double *gmax, double *qmax) {
   for (pic_ctx *c : g->ctx) {
-    cudaMemsetAsync(c->Q, 0, c->grid_elems * sizeof(double), g->stream);
-    cudaMemsetAsync(c->Qa, 0, c->grid_elems * sizeof(double), g->stream);
-    if (c->d.precision == PIC_FP32) charge32(c, c->Q, c->Qa);
-    else charge64(c, c->Q, c->Qa);
+    if (c->d.precision == PIC_FP32) charge32(c);
+    else charge64(c);
   }
   for (int s = 0; s + 1 < g->S; ++s) {
     int e;
@@ -360,7 +358,7 @@ int slab_gauss(pic_slabs *g, bool snapshot, double *gmax, double *qmax) {
   *qmax = 0.0;
   for (int s = 0; s < g->S; ++s) {
     pic_ctx *c = g->ctx[s];
-    filter_array(c, c->Q, c->Qt, 0, +1, g->d.n_filt);
+    filter_charge(c);
     cudaMemsetAsync(c->d_cnt + CNT_GMAX, 0, 2 * sizeof(long long), g->stream);
     const int ilo = std::max(1 - c->G.i0, 0);
     const int ihi = std::min(top - c->G.i0, c->G.open_hi ? c->G.nr - 1 : c->G.nr);
