@@ -15,13 +15,14 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libpicsar_gb300.so")
-SOURCES = ["api.cu", "ensemble.cu", "fields.cu", "particles64.cu", "particles32.cu", "noalloc.cu", "slabs.cu"]
+SOURCES = ["api.cu", "ensemble.cu", "fields.cu", "particles64.cu", "particles32.cu", "tiles_one.cu",
+           "tiles_two.cu", "noalloc.cu", "slabs.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # The FP32 particle kernel takes approximate division and square root (within
 # 2 ulp) and flushes denormals: 5% faster, and the FP32 parity tests against the
 # oracle hold unchanged.  Full --use_fast_math is not used: its sin/cos move
 # positions near the poles by ~1e-5 cell.
-EXTRA = {"particles32.cu": ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]}
+EXTRA = {f: ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"] for f in ("particles32.cu", "tiles_one.cu", "tiles_two.cu")}
 
 
 def _nvcc() -> str:

@@ -232,9 +232,10 @@ int alloc_parts(pic_ctx *c, int64_t cap) {
     Parts32 *a[2] = {&c->p32, &c->q32};
     for (Parts32 *p : a) {
       int e;
-      if ((e = dalloc(&p->cell, n)) || (e = dalloc(&p->dx, n)) || (e = dalloc(&p->dy, n)) ||
-          (e = dalloc(&p->ur, n)) || (e = dalloc(&p->ut, n)) || (e = dalloc(&p->up, n)) ||
-          (e = dalloc(&p->qw, n)) || (e = dalloc(&p->id, n)))
+      // (one slot more: the tile kernel reads slots in pairs)
+      if ((e = dalloc(&p->cell, n + 1)) || (e = dalloc(&p->dx, n + 1)) || (e = dalloc(&p->dy, n + 1)) ||
+          (e = dalloc(&p->ur, n + 1)) || (e = dalloc(&p->ut, n + 1)) || (e = dalloc(&p->up, n + 1)) ||
+          (e = dalloc(&p->qw, n + 1)) || (e = dalloc(&p->id, n)))
         return e;
     }
     PIC_CUDA(cudaMemset(c->p32.qw, 0, n * sizeof(float)));
@@ -571,7 +572,12 @@ int pic_create_context(pic_ctx **out, const pic_desc &d, void *stream, int i0, i
     {
       std::vector<float> rn(d.nr + 2 * G.PI + 1);
       // f_r of each padded row (global rows: a radial slab starts at row i0)
-      for (size_t ii = 0; ii < rn.size(); ++ii) rn[ii] = (float)h_fr(d, G.dxi, (double)ii - G.PI + G.i0);
+      std::vector<float> irn(rn.size());
+      for (size_t ii = 0; ii < rn.size(); ++ii) {
+        const double r = h_fr(d, G.dxi, (double)ii - G.PI + G.i0);
+        rn[ii] = (float)r;
+        irn[ii] = (float)(d.r_map == PIC_R_LOG ? 1.0 / r : r);
+      }
       // The grid bounds the arguments of the move's series: dx dxi <= dxi for
       // exp; with eps = dt / r(-g) (speed < c) the relative displacement s <=
       // 2 eps + 3 eps^2 for log1p and the turning angle below eps for atan and
@@ -583,6 +589,8 @@ int pic_create_context(pic_ctx **out, const pic_desc &d, void *stream, int i0, i
       c->small_steps = d.r_map == PIC_R_LOG && G.dxi <= 1.0 / 16 && G.dt / h_fr(d, G.dxi, -G.g) <= 1.0 / 40;
       if ((e = dalloc(&c->r_n32, rn.size()))) return fail(e);
       PIC_CUDA(cudaMemcpy(c->r_n32, rn.data(), rn.size() * sizeof(float), cudaMemcpyHostToDevice));
+      if ((e = dalloc(&c->ir_n32, irn.size()))) return fail(e);
+      PIC_CUDA(cudaMemcpy(c->ir_n32, irn.data(), irn.size() * sizeof(float), cudaMemcpyHostToDevice));
       std::vector<float2> tn(G.LD);
       for (int jj = 0; jj < G.LD; ++jj) {
         const double2 a = node_angle(jj);
@@ -1107,6 +1115,7 @@ extern "C" int pic_destroy(pic_ctx *c) {
   cudaFree(c->metric_buf);
   for (int k = 0; k < 6; ++k) { cudaFree(c->f[k]); cudaFree(c->f32[k]); }
   cudaFree(c->r_n32);
+  cudaFree(c->ir_n32);
   cudaFree(c->th_n32);
   cudaFree(c->th_n64);
   cudaFree(c->d_tile_maps);

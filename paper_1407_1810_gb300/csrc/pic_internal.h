@@ -146,6 +146,7 @@ struct pic_ctx {
   double *Ft[3] = {};     // FP64 path: the deposit; FP32 path: scratch of a pass-by-pass filter
   float *f32[6] = {};     // FP32 gather copies (FP32 path)
   float *r_n32 = nullptr; // f_r(i) per padded row, FP32 (FP32 path)
+  float *ir_n32 = nullptr; // 1 / f_r(i) (log r) or f_r(i) (linear r)
   float2 *th_n32 = nullptr; // (sin, cos) of the linear map's node angle per padded column (FP32 path)
   double2 *th_n64 = nullptr; // the same in FP64 (FP64 path)
   long long *acc[3] = {}; // fixed-point flux accumulators (FP32 path)
@@ -228,8 +229,8 @@ void ens_inject_smooth(const EnsFieldArg *tab, const EnsList &L, int blocks, int
 void ens_inject_write(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
 // particles32.cu
 int tiles32_setup(pic_ctx *c);         // tensor maps of the field window (FP32 path, at creation)
-// batched tile kernel: members grouped by kind (specialisation x tile shape)
-constexpr int ENS_TILE_KINDS = 9;
+// batched tile kernel: members grouped by kind (form x specialisation x tile shape)
+constexpr int ENS_TILE_KINDS = 18;
 size_t ens_tile_arg_bytes();
 int ens_tile_kind(const pic_ctx *c);
 int64_t ens_tile_blocks(const pic_ctx *c);           // 0 when the member holds no particles
