@@ -103,15 +103,36 @@ int dalloc(T **p, size_t n) {
   return PIC_OK;
 }
 
+// Arrays carved out of one device allocation, each on a 256-byte boundary: a
+// context holds some sixty, and allocating and freeing them one by one took
+// 3.7 ms of a 10.6 ms run.
+struct Block {
+  struct Item { void **p; size_t bytes; };
+  std::vector<Item> items;
+  size_t bytes = 0;
+  template <typename T>
+  void add(T **p, size_t n) {
+    items.push_back({(void **)p, bytes});
+    bytes += (n * sizeof(T) + 255) / 256 * 256;
+  }
+  int allocate(void **block, bool zero) {
+    PIC_CUDA(cudaMalloc(block, std::max<size_t>(bytes, 256)));
+    if (zero) PIC_CUDA(cudaMemset(*block, 0, bytes));
+    for (const Item &i : items) *i.p = (char *)*block + i.bytes;
+    return PIC_OK;
+  }
+};
+
 // ---- metric tables ----------------------------------------------------------
-int build_metric(pic_ctx *c) {
+constexpr int METRIC_ROWS = 21, METRIC_COLS = 18;  // row and column tables
+std::vector<double> build_metric(const pic_ctx *c) {
   const pic_desc &d = c->d;
-  Grid &G = c->G;
+  const Grid &G = c->G;
   const int NRr = d.nr + 2 * G.PI + 1, NC = G.LD;
   const int nrg = G.nr_glob;  // rows of the whole grid (a slab's tables hold its global rows)
   // row tables 0-12 (geometry) and 13-20 (update coefficients); column
   // tables 0-11 and 17 (geometry) and 12-16 (update coefficients)
-  const int nrow = 21, ncol = 18;
+  const int nrow = METRIC_ROWS, ncol = METRIC_COLS;
   const double hh = 0.5 * G.dt, dt = G.dt;
   std::vector<double> h((size_t)nrow * NRr + (size_t)ncol * NC, 0.0);
   auto row = [&](int t) { return h.data() + (size_t)t * NRr; };
@@ -180,9 +201,14 @@ int build_metric(pic_ctx *c) {
       col(15)[cc] = stbm * col(9)[cc];
     }
   }
-  PIC_CUDA(cudaMalloc((void **)&c->metric_buf, h.size() * sizeof(double)));
-  PIC_CUDA(cudaMemcpy(c->metric_buf, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice));
-  const double *R = c->metric_buf, *C = c->metric_buf + (size_t)nrow * NRr;
+  return h;
+}
+
+// the tables' device pointers
+void metric_pointers(pic_ctx *c) {
+  Grid &G = c->G;
+  const int NRr = c->d.nr + 2 * G.PI + 1, NC = G.LD;
+  const double *R = c->metric_buf, *C = c->metric_buf + (size_t)METRIC_ROWS * NRr;
   auto dr = [&](int t) { return R + (size_t)t * NRr; };
   auto dc = [&](int t) { return C + (size_t)t * NC; };
   Metric &m = G.m;
@@ -196,53 +222,40 @@ int build_metric(pic_ctx *c) {
   m.eR = dr(17); m.w0 = dr(18); m.w1 = dr(19); m.wd = dr(20);
   m.cB1 = dc(12); m.cB2 = dc(13); m.cE1 = dc(14); m.cE2 = dc(15); m.cF = dc(16);
   m.cos_tb = dc(17);
-  return PIC_OK;
 }
 
 // ---- particle buffers ----------------------------------------------------------
 void free_parts(pic_ctx *c) {
-  Parts64 *a[2] = {&c->p64, &c->q64};
-  for (Parts64 *p : a) {
-    cudaFree(p->x1); cudaFree(p->x2); cudaFree(p->ur); cudaFree(p->ut); cudaFree(p->up); cudaFree(p->qw);
-    cudaFree(p->id);
-    *p = Parts64{};
-  }
-  Parts32 *b[2] = {&c->p32, &c->q32};
-  for (Parts32 *p : b) {
-    cudaFree(p->cell); cudaFree(p->dx); cudaFree(p->dy); cudaFree(p->ur); cudaFree(p->ut); cudaFree(p->up);
-    cudaFree(p->qw); cudaFree(p->id);
-    *p = Parts32{};
-  }
-  cudaFree(c->scratch);
+  cudaFree(c->parts_block);
+  c->parts_block = nullptr;
+  c->p64 = c->q64 = Parts64{};
+  c->p32 = c->q32 = Parts32{};
   c->scratch = nullptr;
 }
 
 int alloc_parts(pic_ctx *c, int64_t cap) {
   const size_t n = (size_t)cap;
+  Block B;
   if (c->d.precision == PIC_FP64) {
-    Parts64 *a[2] = {&c->p64, &c->q64};
-    for (Parts64 *p : a) {
-      int e;
-      if ((e = dalloc(&p->x1, n)) || (e = dalloc(&p->x2, n)) || (e = dalloc(&p->ur, n)) || (e = dalloc(&p->ut, n)) ||
-          (e = dalloc(&p->up, n)) || (e = dalloc(&p->qw, n)) || (e = dalloc(&p->id, n)))
-        return e;
+    for (Parts64 *p : {&c->p64, &c->q64}) {
+      for (double **a : {&p->x1, &p->x2, &p->ur, &p->ut, &p->up, &p->qw}) B.add(a, n);
+      B.add(&p->id, n);
     }
-    PIC_CUDA(cudaMemset(c->p64.qw, 0, n * sizeof(double)));
   } else {
-    Parts32 *a[2] = {&c->p32, &c->q32};
-    for (Parts32 *p : a) {
-      int e;
-      // (one slot more: the tile kernel reads slots in pairs)
-      if ((e = dalloc(&p->cell, n + 1)) || (e = dalloc(&p->dx, n + 1)) || (e = dalloc(&p->dy, n + 1)) ||
-          (e = dalloc(&p->ur, n + 1)) || (e = dalloc(&p->ut, n + 1)) || (e = dalloc(&p->up, n + 1)) ||
-          (e = dalloc(&p->qw, n + 1)) || (e = dalloc(&p->id, n)))
-        return e;
+    // (one slot more: the tile kernel reads slots in pairs)
+    for (Parts32 *p : {&c->p32, &c->q32}) {
+      B.add(&p->cell, n + 1);
+      for (float **a : {&p->dx, &p->dy, &p->ur, &p->ut, &p->up, &p->qw}) B.add(a, n + 1);
+      B.add(&p->id, n);
     }
-    PIC_CUDA(cudaMemset(c->p32.qw, 0, n * sizeof(float)));
   }
   // scratch: block counts of the FP64 path's stable compaction
   c->scratch_bytes = ((size_t)cap / 256 + 2) * sizeof(long long);
-  PIC_CUDA(cudaMalloc(&c->scratch, c->scratch_bytes));
+  B.add((char **)&c->scratch, c->scratch_bytes);
+  const int e = B.allocate(&c->parts_block, false);
+  if (e) return e;
+  if (c->d.precision == PIC_FP64) PIC_CUDA(cudaMemset(c->p64.qw, 0, n * sizeof(double)));
+  else PIC_CUDA(cudaMemset(c->p32.qw, 0, n * sizeof(float)));
   c->cap = cap;
   return PIC_OK;
 }
@@ -277,42 +290,106 @@ int grow_parts(pic_ctx *c, int64_t new_cap) {
   free_parts(c);
   c->p64 = tmp.p64; c->q64 = tmp.q64; c->p32 = tmp.p32; c->q32 = tmp.q32;
   c->scratch = tmp.scratch; c->scratch_bytes = tmp.scratch_bytes;
+  c->parts_block = tmp.parts_block;
   c->cap = new_cap;
-  tmp.p64 = tmp.q64 = Parts64{};
-  tmp.p32 = tmp.q32 = Parts32{};
-  tmp.scratch = nullptr;
   return PIC_OK;
 }
 
 int64_t inject_slots(const pic_ctx *c) { return c->d.inject ? (int64_t)2 * c->d.pairs_per_cell * c->d.nth : 0; }
 
+int to_user(pic_ctx *c, const double *dsrc, double *out, size_t n, int mem) {
+  PIC_CUDA(cudaMemcpyAsync(out, dsrc, n * sizeof(double),
+                           mem == PIC_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
+  PIC_CUDA(cudaStreamSynchronize(c->stream));
+  return PIC_OK;
+}
+
 // ---- layout conversion between the padded arrays and the dense API planes ----
-__global__ void k_pack(Grid G, const double *__restrict__ src, double *__restrict__ dst, int i_lo, int rows, int cols,
-                       int imax, int jmax, int unpack) {
+// Up to six planes at once, each rows x cols from row i_lo on; entries outside
+// a component's range are 0 (left alone when unpacking)
+struct Planes {
+  double *src[6];
+  int imax[6], jmax[6];
+  int n;
+};
+__global__ void k_pack(Grid G, Planes S, double *dst, int i_lo, int rows, int cols, int unpack) {
   const int j = blockIdx.x * 32 + threadIdx.x, r = blockIdx.y * 8 + threadIdx.y;
   if (r >= rows || j >= cols) return;
   const int i = i_lo + r;
-  const size_t o = gidx(G, i, j), q = (size_t)r * cols + j;
-  const bool in = i <= imax && j <= jmax;
-  if (unpack) { if (in) ((double *)src)[o] = dst[q]; }
-  else dst[q] = in ? src[o] : 0.0;
+  const size_t o = gidx(G, i, j), plane = (size_t)rows * cols, q = (size_t)r * cols + j;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    if (k >= S.n) break;
+    const bool in = i <= S.imax[k] && j <= S.jmax[k];
+    if (unpack) { if (in) S.src[k][o] = dst[k * plane + q]; }
+    else dst[k * plane + q] = in ? S.src[k][o] : 0.0;
+  }
 }
 
-// plasma plus analytic field of component k at its staggered points, time t
-__global__ void k_pack_total(Grid G, const double *__restrict__ src, double *__restrict__ dst, int k, int rows,
-                             int cols, int imax, int jmax, double t) {
+// plasma plus analytic field of the six components at their staggered points, time t
+__global__ void k_pack_total(Grid G, Planes S, double *__restrict__ dst, int rows, int cols, double t) {
   const int j = blockIdx.x * 32 + threadIdx.x, i = blockIdx.y * 8 + threadIdx.y;
   if (i >= rows || j >= cols) return;
-  const size_t q = (size_t)i * cols + j;
-  if (i > imax || j > jmax) { dst[q] = 0.0; return; }
+  const size_t plane = (size_t)rows * cols, q = (size_t)i * cols + j;
   const Metric &m = G.m;
-  const double r = stag_i(k) ? m.r_h[i + G.PI] : m.r_n[i + G.PI];
-  const double st = stag_j(k) ? m.sin_tb[j + G.PJ] : m.sin_t[j + G.PJ];
-  const double ct = stag_j(k) ? m.cos_tb[j + G.PJ] : m.cos_t[j + G.PJ];
-  double E[3], B[3];
   const Vac<double> V{G.vacuum, G.b0, G.r_min, omega_at(G.omega, G.t_spin, t)};
-  vacuum_field<double>(V, r, st, ct, false, E, B);
-  dst[q] = src[gidx(G, i, j)] + (k < 3 ? E[k] : B[k - 3]);
+  for (int k = 0; k < 6; ++k) {
+    if (i > S.imax[k] || j > S.jmax[k]) { dst[k * plane + q] = 0.0; continue; }
+    const double r = stag_i(k) ? m.r_h[i + G.PI] : m.r_n[i + G.PI];
+    const double st = stag_j(k) ? m.sin_tb[j + G.PJ] : m.sin_t[j + G.PJ];
+    const double ct = stag_j(k) ? m.cos_tb[j + G.PJ] : m.cos_t[j + G.PJ];
+    double E[3], B[3];
+    vacuum_field<double>(V, r, st, ct, false, E, B);
+    dst[k * plane + q] = S.src[k][gidx(G, i, j)] + (k < 3 ? E[k] : B[k - 3]);
+  }
+}
+
+Planes field_planes(const pic_ctx *c) {
+  Planes S;
+  S.n = 6;
+  for (int k = 0; k < 6; ++k) {
+    S.src[k] = c->f[k];
+    S.imax[k] = stag_i(k) ? c->d.nr - 1 : c->d.nr;
+    S.jmax[k] = stag_j(k) ? c->d.nth - 1 : c->d.nth;
+  }
+  return S;
+}
+
+// Whether a kernel can write n doubles at `out` itself: memory of the GPU
+// (or managed), on an 8-byte boundary.  Anything else takes a staging copy.
+bool writable_here(const pic_ctx *c, const void *out, int mem) {
+  if (mem != PIC_MEM_DEVICE || ((uintptr_t)out & 7) != 0) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, out) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (a.type == cudaMemoryTypeDevice && a.device == c->device) || a.type == cudaMemoryTypeManaged;
+}
+
+// Runs `fill(double *dst)` (kernels that write n doubles) into the caller's
+// buffer: directly where a kernel can write there, otherwise through the
+// context's staging area or, for more than it holds, an allocation; and waits
+// for it.  (A 250 x 231 grid's fields to the device: 246 us with an allocation,
+// six launches, a copy and a free, 44 us so.)
+template <class Fill>
+int deliver(pic_ctx *c, double *out, size_t n, int mem, const Fill &fill) {
+  if (writable_here(c, out, mem)) {
+    fill(out);
+    PIC_CUDA(cudaGetLastError());
+    PIC_CUDA(cudaStreamSynchronize(c->stream));
+    return PIC_OK;
+  }
+  if (n <= c->stage_elems) {
+    fill(c->stage);
+    return to_user(c, c->stage, out, n, mem);
+  }
+  double *tmp;
+  PIC_CUDA(cudaMalloc((void **)&tmp, n * sizeof(double)));
+  fill(tmp);
+  const int e = to_user(c, tmp, out, n, mem);
+  cudaFree(tmp);
+  return e;
 }
 
 __global__ void k_grid_coords(Grid G, int64_t n, const double *__restrict__ r, const double *__restrict__ th,
@@ -321,13 +398,6 @@ __global__ void k_grid_coords(Grid G, int64_t n, const double *__restrict__ r, c
   if (k >= n) return;
   x1[k] = map_r_inv(G, r[k]);
   x2[k] = map_th_inv(G, th[k]);
-}
-
-int to_user(pic_ctx *c, const double *dsrc, double *out, size_t n, int mem) {
-  PIC_CUDA(cudaMemcpyAsync(out, dsrc, n * sizeof(double),
-                           mem == PIC_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
-  PIC_CUDA(cudaStreamSynchronize(c->stream));
-  return PIC_OK;
 }
 
 int latch_errors(pic_ctx *c) {
@@ -482,11 +552,14 @@ static int alloc_bins(pic_ctx *c, int shape) {
   T.ntiles = T.nti * T.ntj;
   T.nbins = (int64_t)T.ntiles * T.tc + 1;
   const int64_t nblk = T.nbins / SCAN_CHUNK + 2;
-  int e;
-  if ((e = dalloc(&T.start, (size_t)T.nbins + 1)) || (e = dalloc(&T.cursor, (size_t)T.nbins + 1)) ||
-      (e = dalloc(&T.bsum, 2 * (size_t)nblk)) || (e = dalloc(&T.ucount, (size_t)T.ntiles + 1)) ||
-      (e = dalloc(&T.usum, 2 * ((size_t)T.ntiles / SCAN_CHUNK + 2))))
-    return e;
+  Block B;
+  B.add(&T.start, (size_t)T.nbins + 1);
+  B.add(&T.cursor, (size_t)T.nbins + 1);
+  B.add(&T.bsum, 2 * (size_t)nblk);
+  B.add(&T.ucount, (size_t)T.ntiles + 1);
+  B.add(&T.usum, 2 * ((size_t)T.ntiles / SCAN_CHUNK + 2));
+  const int e = B.allocate(&T.block, false);
+  if (e) return e;
   PIC_CUDA(cudaMemset(T.start, 0, (T.nbins + 1) * sizeof(int64_t)));
   return PIC_OK;
 }
@@ -524,98 +597,94 @@ int pic_create_context(pic_ctx **out, const pic_desc &d, void *stream, int i0, i
   c->grid_elems = (size_t)(d.nr + 2 * G.PI + 1) * G.LD;
   const size_t ge = c->grid_elems;
   auto fail = [&](int code) { pic_destroy(c); return code; };
-  if ((e = build_metric(c))) return fail(e);
-  for (int k = 0; k < 6; ++k)
-    if ((e = dalloc(&c->f[k], ge))) return fail(e);
-  for (int k = 0; k < 3; ++k)
-    if ((e = dalloc(&c->F[k], ge)) || (e = dalloc(&c->Ft[k], ge)) || (e = dalloc(&c->bh[k], ge))) return fail(e);
-  if ((e = dalloc(&c->Q, ge)) || (e = dalloc(&c->Qa, ge)) || (e = dalloc(&c->Qt, ge)) || (e = dalloc(&c->gsnap, ge)))
-    return fail(e);
-  for (int k = 0; k < 6; ++k) cudaMemset(c->f[k], 0, ge * 8);
+  const bool fp32 = d.precision == PIC_FP32;
+  const std::vector<double> metric = build_metric(c);
+  const size_t nrp = (size_t)d.nr + 2 * G.PI + 1;
+  Block B;
+  B.add(&c->metric_buf, metric.size());
+  for (int k = 0; k < 6; ++k) B.add(&c->f[k], ge);
   for (int k = 0; k < 3; ++k) {
-    cudaMemset(c->F[k], 0, ge * 8);
-    cudaMemset(c->Ft[k], 0, ge * 8);
-    cudaMemset(c->bh[k], 0, ge * 8);
+    B.add(&c->F[k], ge);
+    B.add(&c->Ft[k], ge);
+    B.add(&c->bh[k], ge);
+    if (lossy_first_row(c) >= 0)  // E of the lossy rows before the layer acts
+      B.add(&c->epre[k], (size_t)(d.nr + 1 - lossy_first_row(c)) * G.LD);
   }
-  c->bh_ok = true;  // no field yet
-  if (lossy_first_row(c) >= 0) {  // E of the lossy rows before the layer acts
-    const size_t n = (size_t)(d.nr + 1 - lossy_first_row(c)) * G.LD;
-    for (int k = 0; k < 3; ++k) {
-      if ((e = dalloc(&c->epre[k], n))) return fail(e);
-      cudaMemset(c->epre[k], 0, n * 8);
-    }
+  for (double **p : {&c->Q, &c->Qa, &c->Qt, &c->gsnap}) B.add(p, ge);
+  if (fp32) {
+    for (int k = 0; k < 6; ++k) B.add(&c->f32[k], ge);
+    for (int k = 0; k < 3; ++k) B.add(&c->acc[k], ge);
+    B.add(&c->r_n32, nrp);
+    B.add(&c->ir_n32, nrp);
+    B.add(&c->th_n32, (size_t)G.LD);
+    B.add(&c->d_tile_maps, sizeof c->tile_maps);
+  } else {
+    B.add(&c->th_n64, (size_t)G.LD);
   }
-  cudaMemset(c->Q, 0, ge * 8); cudaMemset(c->Qa, 0, ge * 8); cudaMemset(c->Qt, 0, ge * 8);
-  cudaMemset(c->gsnap, 0, ge * 8);
-  // sine and cosine of the node angle pi j / nth of the linear theta map at
-  // padded column jj, each the sine of an angle measured from the nearer pole
-  // or from the equator (exact zeros and ones at the poles and the equator)
-  auto node_angle = [&](int jj) {
-    const double j = (double)(jj - G.PJ), m = std::min(j, d.nth - j);
-    return make_double2(std::sin(M_PI * m / d.nth), std::sin(M_PI * (d.nth - 2.0 * j) / (2.0 * d.nth)));
+  // staging of a small grid's readout to the host (12 MB at most)
+  const size_t dense = 6 * (size_t)(d.nr + 2 * G.g + 1) * (d.nth + 1);
+  c->stage_elems = dense <= 6 * (size_t)(1 << 18) ? dense : 0;
+  B.add(&c->stage, c->stage_elems);
+  B.add(&c->sig, 2 * ((size_t)d.nth + 1));
+  B.add(&c->d_err, 1);
+  B.add(&c->d_cnt, CNT_N);
+  B.add(&c->d_acc, ACC_N);
+  B.add(&c->tie_step, TIE_LOG);
+  B.add(&c->tie_id, TIE_LOG);
+  B.add(&c->tie_sign, TIE_LOG);
+  if ((e = B.allocate(&c->block, true))) return fail(e);
+  metric_pointers(c);
+  auto upload = [&](void *dst, const void *src, size_t bytes) {
+    return cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess
+               ? PIC_OK : pic_fail(PIC_ECUDA, "context tables");
   };
-  if (d.precision == PIC_FP64) {
-    std::vector<double2> tn(G.LD);
-    for (int jj = 0; jj < G.LD; ++jj) tn[jj] = node_angle(jj);
-    if ((e = dalloc(&c->th_n64, tn.size()))) return fail(e);
-    PIC_CUDA(cudaMemcpy(c->th_n64, tn.data(), tn.size() * sizeof(double2), cudaMemcpyHostToDevice));
+  if ((e = upload(c->metric_buf, metric.data(), metric.size() * sizeof(double)))) return fail(e);
+  c->bh_ok = true;  // no field yet
+  // sine and cosine of the node angle pi j / nth of the linear theta map per
+  // padded column, each the sine of an angle measured from the nearer pole
+  // or from the equator (exact zeros and ones at the poles and the equator);
+  // FP32: rounded once
+  std::vector<double2> tn(G.LD);
+  for (int jj = 0; jj < G.LD; ++jj) {
+    const double j = (double)(jj - G.PJ), m = std::min(j, d.nth - j);
+    tn[jj] = make_double2(std::sin(M_PI * m / d.nth), std::sin(M_PI * (d.nth - 2.0 * j) / (2.0 * d.nth)));
   }
-  if (d.precision == PIC_FP32) {
-    for (int k = 0; k < 6; ++k) {
-      if ((e = dalloc(&c->f32[k], ge))) return fail(e);
-      cudaMemset(c->f32[k], 0, ge * 4);
+  if (!fp32) {
+    if ((e = upload(c->th_n64, tn.data(), tn.size() * sizeof(double2)))) return fail(e);
+  } else {
+    std::vector<float2> tf(tn.size());
+    for (size_t k = 0; k < tn.size(); ++k) tf[k] = make_float2((float)tn[k].x, (float)tn[k].y);
+    // f_r of each padded row (global rows: a radial slab starts at row i0)
+    std::vector<float> rn(nrp), irn(nrp);
+    for (size_t ii = 0; ii < nrp; ++ii) {
+      const double r = h_fr(d, G.dxi, (double)ii - G.PI + G.i0);
+      rn[ii] = (float)r;
+      irn[ii] = (float)(d.r_map == PIC_R_LOG ? 1.0 / r : r);
     }
-    for (int k = 0; k < 3; ++k) {
-      if ((e = dalloc(&c->acc[k], ge))) return fail(e);
-      cudaMemset(c->acc[k], 0, ge * 8);
-    }
-    {
-      std::vector<float> rn(d.nr + 2 * G.PI + 1);
-      // f_r of each padded row (global rows: a radial slab starts at row i0)
-      std::vector<float> irn(rn.size());
-      for (size_t ii = 0; ii < rn.size(); ++ii) {
-        const double r = h_fr(d, G.dxi, (double)ii - G.PI + G.i0);
-        rn[ii] = (float)r;
-        irn[ii] = (float)(d.r_map == PIC_R_LOG ? 1.0 / r : r);
-      }
-      // The grid bounds the arguments of the move's series: dx dxi <= dxi for
-      // exp; with eps = dt / r(-g) (speed < c) the relative displacement s <=
-      // 2 eps + 3 eps^2 for log1p and the turning angle below eps for atan and
-      // the sin / cos series.  With dxi <= 1/16 and eps <= 1/40 every series'
-      // relative truncation stays below 2^-28, 1/16 of an FP32 ulp (at the
-      // bounds, evaluated in FP64: exp 8.8e-11, log1p 2.9e-9, atan and the
-      // sin / cos series below 1e-13), so the step uses the series without
-      // the general fallback
-      c->small_steps = d.r_map == PIC_R_LOG && G.dxi <= 1.0 / 16 && G.dt / h_fr(d, G.dxi, -G.g) <= 1.0 / 40;
-      if ((e = dalloc(&c->r_n32, rn.size()))) return fail(e);
-      PIC_CUDA(cudaMemcpy(c->r_n32, rn.data(), rn.size() * sizeof(float), cudaMemcpyHostToDevice));
-      if ((e = dalloc(&c->ir_n32, irn.size()))) return fail(e);
-      PIC_CUDA(cudaMemcpy(c->ir_n32, irn.data(), irn.size() * sizeof(float), cudaMemcpyHostToDevice));
-      std::vector<float2> tn(G.LD);
-      for (int jj = 0; jj < G.LD; ++jj) {
-        const double2 a = node_angle(jj);
-        tn[jj] = make_float2((float)a.x, (float)a.y);
-      }
-      if ((e = dalloc(&c->th_n32, tn.size()))) return fail(e);
-      PIC_CUDA(cudaMemcpy(c->th_n32, tn.data(), tn.size() * sizeof(float2), cudaMemcpyHostToDevice));
-    }
+    // The grid bounds the arguments of the move's series: dx dxi <= dxi for
+    // exp; with eps = dt / r(-g) (speed < c) the relative displacement s <=
+    // 2 eps + 3 eps^2 for log1p and the turning angle below eps for atan and
+    // the sin / cos series.  With dxi <= 1/16 and eps <= 1/40 every series'
+    // relative truncation stays below 2^-28, 1/16 of an FP32 ulp (at the
+    // bounds, evaluated in FP64: exp 8.8e-11, log1p 2.9e-9, atan and the
+    // sin / cos series below 1e-13), so the step uses the series without
+    // the general fallback
+    c->small_steps = d.r_map == PIC_R_LOG && G.dxi <= 1.0 / 16 && G.dt / h_fr(d, G.dxi, -G.g) <= 1.0 / 40;
+    if ((e = upload(c->th_n32, tf.data(), tf.size() * sizeof(float2))) ||
+        (e = upload(c->r_n32, rn.data(), nrp * sizeof(float))) ||
+        (e = upload(c->ir_n32, irn.data(), nrp * sizeof(float))))
+      return fail(e);
     c->tiles.row0 = -G.g;
     if ((e = alloc_bins(c, d.tile_shape))) return fail(e);
     if (tiles32_setup(c)) return fail(pic_fail(PIC_ECUDA, "tensor maps of the field window could not be encoded"));
   }
-  if ((e = dalloc(&c->sig, 2 * ((size_t)d.nth + 1)))) return fail(e);
-  if ((e = dalloc(&c->d_err, 1)) || (e = dalloc(&c->d_cnt, CNT_N)) || (e = dalloc(&c->d_acc, ACC_N))) return fail(e);
-  cudaMemset(c->d_err, 0, sizeof(int));
-  cudaMemset(c->d_cnt, 0, CNT_N * sizeof(long long));
   c->qexp = c->d_cnt + CNT_QEXP;
   {  // fixed-point exponent: raised on the device by the charges loaded or injected
     long long q0 = QEXP_NONE;
     if (d.flux_quantum > 0.0)
       q0 = std::min<long long>(QEXP_MAX, std::max<long long>(QEXP_MIN, (long long)std::ceil(std::log2(d.flux_quantum)) + KFIX));
-    PIC_CUDA(cudaMemcpy(c->qexp, &q0, sizeof q0, cudaMemcpyHostToDevice));
+    if ((e = upload(c->qexp, &q0, sizeof q0))) return fail(e);
   }
-  if ((e = dalloc(&c->tie_step, TIE_LOG)) || (e = dalloc(&c->tie_id, TIE_LOG)) || (e = dalloc(&c->tie_sign, TIE_LOG)))
-    return fail(e);
   PIC_CUDA(cudaMallocHost((void **)&c->h_pinned, 64));
   PIC_CUDA(cudaDeviceSynchronize());
   *out = c;
@@ -784,19 +853,13 @@ extern "C" int pic_get_fields(pic_ctx *c, int32_t which, double *out6, int64_t *
   const size_t plane = (size_t)rows * cols;
   *n = (int64_t)(6 * plane);
   if (!out6) return PIC_OK;
-  double *tmp;
-  PIC_CUDA(cudaMalloc((void **)&tmp, 6 * plane * sizeof(double)));
-  dim3 gr((cols + 31) / 32, (rows + 7) / 8);
-  for (int k = 0; k < 6; ++k) {
-    int imax = stag_i(k) ? c->d.nr - 1 : c->d.nr, jmax = stag_j(k) ? c->d.nth - 1 : c->d.nth;
-    if (which == PIC_FIELDS_TOTAL)
-      ++c->launches, k_pack_total<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, c->f[k], tmp + k * plane, k, rows, cols, imax,
-                                                                     jmax, c->step * c->G.dt);
-    else
-      ++c->launches, k_pack<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, c->f[k], tmp + k * plane, 0, rows, cols, imax, jmax, 0);
-  }
-  int e = to_user(c, tmp, out6, 6 * plane, mem);
-  cudaFree(tmp);
+  const dim3 gr((cols + 31) / 32, (rows + 7) / 8), bl(32, 8);
+  const Planes S = field_planes(c);
+  const int e = deliver(c, out6, 6 * plane, mem, [&](double *dst) {
+    ++c->launches;
+    if (which == PIC_FIELDS_TOTAL) k_pack_total<<<gr, bl, 0, c->stream>>>(c->G, S, dst, rows, cols, c->step * c->G.dt);
+    else k_pack<<<gr, bl, 0, c->stream>>>(c->G, S, dst, 0, rows, cols, 0);
+  });
   if (e) return e;
   latch_errors(c);
   return status(c);
@@ -811,10 +874,7 @@ extern "C" int pic_set_fields(pic_ctx *c, const double *in6, int32_t mem) {
   PIC_CUDA(cudaMemcpyAsync(tmp, in6, 6 * plane * sizeof(double),
                            mem == PIC_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
   dim3 gr((cols + 31) / 32, (rows + 7) / 8);
-  for (int k = 0; k < 6; ++k) {
-    int imax = stag_i(k) ? c->d.nr - 1 : c->d.nr, jmax = stag_j(k) ? c->d.nth - 1 : c->d.nth;
-    ++c->launches, k_pack<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, c->f[k], tmp + k * plane, 0, rows, cols, imax, jmax, 1);
-  }
+  ++c->launches, k_pack<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, field_planes(c), tmp, 0, rows, cols, 1);
   fields_fill_ghosts(c);
   PIC_CUDA(cudaStreamSynchronize(c->stream));
   cudaFree(tmp);
@@ -829,15 +889,17 @@ extern "C" int pic_get_flux(pic_ctx *c, double *out3, int64_t *n, int32_t mem) {
   const size_t plane = (size_t)rows * cols;
   *n = (int64_t)(3 * plane);
   if (!out3) return PIC_OK;
-  double *tmp;
-  PIC_CUDA(cudaMalloc((void **)&tmp, 3 * plane * sizeof(double)));
-  dim3 gr((cols + 31) / 32, (rows + 7) / 8);
-  for (int k = 0; k < 3; ++k)
-    ++c->launches, k_pack<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, c->F[k], tmp + k * plane, -g, rows, cols, c->d.nr + g,
-                                              k == 1 ? c->d.nth - 1 : c->d.nth, 0);
-  int e = to_user(c, tmp, out3, 3 * plane, mem);
-  cudaFree(tmp);
-  return e;
+  Planes S;
+  S.n = 3;
+  for (int k = 0; k < 3; ++k) {
+    S.src[k] = c->F[k];
+    S.imax[k] = c->d.nr + g;
+    S.jmax[k] = k == 1 ? c->d.nth - 1 : c->d.nth;
+  }
+  const dim3 gr((cols + 31) / 32, (rows + 7) / 8);
+  return deliver(c, out3, 3 * plane, mem, [&](double *dst) {
+    ++c->launches, k_pack<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, S, dst, -g, rows, cols, 0);
+  });
 }
 
 extern "C" int pic_get_charge(pic_ctx *c, int32_t filtered, double *out, int64_t *n, int32_t mem) {
@@ -849,12 +911,15 @@ extern "C" int pic_get_charge(pic_ctx *c, int32_t filtered, double *out, int64_t
   if (c->d.precision == PIC_FP32) charge32(c);
   else charge64(c);
   if (filtered) filter_charge(c);
-  double *tmp;
-  PIC_CUDA(cudaMalloc((void **)&tmp, plane * sizeof(double)));
-  dim3 gr((cols + 31) / 32, (rows + 7) / 8);
-  ++c->launches, k_pack<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, c->Q, tmp, -g, rows, cols, c->d.nr + g, c->d.nth, 0);
-  int e = to_user(c, tmp, out, plane, mem);
-  cudaFree(tmp);
+  Planes S;
+  S.n = 1;
+  S.src[0] = c->Q;
+  S.imax[0] = c->d.nr + g;
+  S.jmax[0] = c->d.nth;
+  const dim3 gr((cols + 31) / 32, (rows + 7) / 8);
+  const int e = deliver(c, out, plane, mem, [&](double *dst) {
+    ++c->launches, k_pack<<<gr, dim3(32, 8), 0, c->stream>>>(c->G, S, dst, -g, rows, cols, 0);
+  });
   if (e) return e;
   latch_errors(c);
   return status(c);
@@ -938,12 +1003,7 @@ extern "C" int pic_get_luminosity(pic_ctx *c, double *L, int64_t *n, int32_t mem
   if (!c || !n) return pic_fail(PIC_EINVAL, "null argument");
   *n = c->d.nr + 1;
   if (!L) return PIC_OK;
-  double *tmp;
-  PIC_CUDA(cudaMalloc((void **)&tmp, (size_t)(c->d.nr + 1) * sizeof(double)));
-  luminosity(c, c->step * c->G.dt, tmp);
-  PIC_CUDA(cudaGetLastError());
-  int e = to_user(c, tmp, L, c->d.nr + 1, mem);
-  cudaFree(tmp);
+  const int e = deliver(c, L, (size_t)c->d.nr + 1, mem, [&](double *dst) { luminosity(c, c->step * c->G.dt, dst); });
   if (e) return e;
   latch_errors(c);
   return status(c);
@@ -1059,11 +1119,8 @@ extern "C" int pic_get_launches(pic_ctx *c, int64_t *n) {
 int pic_set_tiles(pic_ctx *c, int shape) {
   Tiles &T = c->tiles;
   cudaStreamSynchronize(c->stream);
-  cudaFree(T.start);
-  cudaFree(T.cursor);
-  cudaFree(T.bsum);
-  cudaFree(T.ucount);
-  cudaFree(T.usum);
+  cudaFree(T.block);
+  T.block = nullptr;
   T.start = T.cursor = T.bsum = T.ucount = T.usum = nullptr;
   T.sorted_end = 0;
   T.nunits = 0;
@@ -1112,19 +1169,9 @@ extern "C" int pic_destroy(pic_ctx *c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
   free_parts(c);
-  cudaFree(c->metric_buf);
-  for (int k = 0; k < 6; ++k) { cudaFree(c->f[k]); cudaFree(c->f32[k]); }
-  cudaFree(c->r_n32);
-  cudaFree(c->ir_n32);
-  cudaFree(c->th_n32);
-  cudaFree(c->th_n64);
-  cudaFree(c->d_tile_maps);
-  for (int k = 0; k < 3; ++k) { cudaFree(c->F[k]); cudaFree(c->Ft[k]); cudaFree(c->acc[k]); cudaFree(c->bh[k]); cudaFree(c->epre[k]); }
-  cudaFree(c->Q); cudaFree(c->Qa); cudaFree(c->Qt); cudaFree(c->gsnap); cudaFree(c->sig);
-  cudaFree(c->d_err); cudaFree(c->d_cnt); cudaFree(c->d_acc);
-  cudaFree(c->tiles.start); cudaFree(c->tiles.cursor); cudaFree(c->tiles.bsum);
-  cudaFree(c->tiles.ucount); cudaFree(c->tiles.usum); cudaFree(c->tiles.units);
-  cudaFree(c->tie_step); cudaFree(c->tie_id); cudaFree(c->tie_sign);
+  cudaFree(c->block);
+  cudaFree(c->tiles.block);
+  cudaFree(c->tiles.units);
   cudaFree(c->hint_step); cudaFree(c->hint_id); cudaFree(c->hint_sign);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);

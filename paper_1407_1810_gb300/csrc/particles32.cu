@@ -583,9 +583,7 @@ int tiles32_setup(pic_ctx *c) {
       encode_maps<32, 8>(c, fn, c->tile_maps[2]))
     return -1;
   // a device copy for the batched ensemble kernel (the arrays never move)
-  if (cudaMalloc((void **)&c->d_tile_maps, sizeof c->tile_maps) != cudaSuccess ||
-      cudaMemcpy(c->d_tile_maps, c->tile_maps, sizeof c->tile_maps, cudaMemcpyHostToDevice) != cudaSuccess)
-    return -1;
+  if (cudaMemcpy(c->d_tile_maps, c->tile_maps, sizeof c->tile_maps, cudaMemcpyHostToDevice) != cudaSuccess) return -1;
   return 0;
 }
 

@@ -74,6 +74,7 @@ struct Tiles {
   int nti = 0, ntj = 0, ntiles = 0;
   int row0 = 0;                   // first tile row (cell index)
   int tc = 256;                   // cells per tile, TI * TJ
+  void *block = nullptr;          // the allocation of the bin arrays below
   int64_t nbins = 0;              // ntiles * tc cell bins + 1 bin of removed particles
   int64_t *start = nullptr;       // nbins + 1 bin starts: tile t is [start[t tc], start[(t+1) tc])
   int64_t *cursor = nullptr;      // nbins + 1 counts, then scatter cursors
@@ -136,6 +137,8 @@ struct pic_ctx {
   cudaStream_t stream = nullptr;
   int device = 0;
   pic::Grid G{};
+  void *block = nullptr;        // the allocation that holds the context's own arrays
+  void *parts_block = nullptr;  // the particle arrays and scratch
   double *metric_buf = nullptr;
   size_t grid_elems = 0;  // elements of one padded grid array
   double *f[6] = {};      // plasma fields (FP64)
@@ -154,6 +157,8 @@ struct pic_ctx {
   unsigned char *d_tile_maps = nullptr;  // the same maps in device memory (batched ensemble launches)
   double *Q = nullptr, *Qa = nullptr, *Qt = nullptr, *gsnap = nullptr;
   bool have_snap = false;
+  double *stage = nullptr;  // staging of readouts (small grids)
+  size_t stage_elems = 0;
   double *sig = nullptr;  // injection: surface charge per cell, two buffers of nth + 1 (smoothing)
   // particles
   int64_t cap = 0, n_used = 0;
