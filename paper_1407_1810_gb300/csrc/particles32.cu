@@ -163,7 +163,7 @@ __global__ void k_scan_apply(int64_t *count, int64_t *start, int64_t nb, const i
   scan_apply_block(count, start, nb, offs, nblk, blockIdx.x);
 }
 
-// work units of each tile: ceil(n_t / unit), none for an empty tile
+// work units of each tile: ceil(n_t / unit) of even size, none for an empty tile
 __device__ __forceinline__ void unit_count_at(int t, const int64_t *start, int tc, int ntiles, int64_t unit,
                                               int64_t *ucount) {
   if (t >= ntiles) return;
@@ -359,10 +359,8 @@ __global__ void __launch_bounds__(NT) k_charge_tiles(Args32 A, Parts32 P, Charge
   int64_t b0, b1;
   int i0 = 0, j0 = 0;
   if (binned) {
-    const long long u = A.units[blk];
-    const int t = (int)(u >> 32);
-    b0 = A.start[(int64_t)t * A.tc] + (u & 0xffffffffll) * A.unit;
-    b1 = min(A.start[(int64_t)(t + 1) * A.tc], b0 + A.unit);
+    int t;
+    unit_range(A, A.units[blk], t, b0, b1);
     if (b1 <= b0) return;
     i0 = A.row0 + (t / A.ntj) * TI;
     j0 = (t % A.ntj) * TJ;
@@ -678,21 +676,42 @@ int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaSt
   return launches;
 }
 
-// Particles per work unit.  A context on its own: no more than about 1216
-// units besides one per tile (two waves of 4 CTAs on each of the 152 SMs), so
-// a large run keeps one unit per tile while the tiles of a small plasma are
-// spread over the chip; and at least two passes of a CTA's threads, below
-// which a CTA's window and flush cost more than its particles.  (72 x 56
-// rotator, 1e5 particles, 20 steps with the fields read out: 0.91 ms with
-// units of 512, 0.96 with 1024, 1.10 with 2048, 1.39 with 4096.)  Members of
-// an ensemble share the chip: their units follow the particles of all of them
-// (64 members, 2.4e7 particles: 62 ms for 40 steps with units of 4096, 64 with
-// 2048, 71 with 1024, 78 with 512).
-constexpr int64_t UNIT_MIN = 2 * NT, UNITS_ALONE = 2 * 4 * 152, UNITS_ENSEMBLE = 8 * 4 * 152;
+// Particles per work unit of a context on its own.  The 152 SMs hold 608 CTAs
+// at a time, so the kernel runs in rounds of 608 units: cutting each tile's
+// bin into m even units takes about ceil(m tiles / 608) rounds of the passes a
+// unit needs and its window and flush, worth 1.5 passes.  The m with the least
+// is taken; the bound is a tenth above the even share, so that a tile a little
+// fuller than the average is not cut once more.  At least 1 / 2432 of the
+// particles: where they crowd in few tiles, four rounds are cut fine enough.
+// (Steps alone, units of 1 / 1216 of the
+// particles -> so: 20 steps of monopole 250 x 231 1.70 -> 1.65 ms, of dipole
+// 192 x 160 1.31 -> 1.20, of rotator 72 x 56 0.84 either way; 19 of monopole
+// 448 x 416 3.56 -> 3.47.)
+// Members of an ensemble share the chip: their units follow the particles of
+// all of them (64 members, 2.4e7 particles: 62 ms for 40 steps with units of
+// 4096, 64 with 2048, 71 with 1024, 78 with 512).
+constexpr int SLOTS = 4 * 152;
 static int64_t unit_size(const pic_ctx *c) {
-  const int64_t n = c->ens_particles > 0 ? c->ens_particles : c->n_used;
-  const int64_t units = c->ens_particles > 0 ? UNITS_ENSEMBLE : UNITS_ALONE;
-  return std::max(UNIT_MIN, ((n + units - 1) / units + NT - 1) / NT * NT);
+  const int64_t n = c->n_used;
+  if (c->ens_particles > 0) {
+    const int64_t u = (c->ens_particles + 8 * SLOTS - 1) / (8 * SLOTS);
+    return std::max<int64_t>(2 * NT, (u + NT - 1) / NT * NT);
+  }
+  const Tiles &T = c->tiles;
+  const int64_t tiles = (int64_t)((c->G.nr + T.TI - 1) / T.TI) * T.ntj;  // those of the grid proper
+  const double avg = (double)n / (double)tiles;
+  double best = 1e300;
+  int64_t unit = NT;
+  for (int m = 1; m <= 64; ++m) {
+    const double share = avg / m;
+    const double cost = std::ceil((double)m * tiles / SLOTS) * (std::ceil(share / NT) + 1.5);
+    if (cost < best) {
+      best = cost;
+      unit = std::max<int64_t>(NT, (int64_t)(1.1 * share) + 1);
+    }
+    if (share <= NT) break;
+  }
+  return std::max(unit, (n + 4 * SLOTS - 1) / (4 * SLOTS));
 }
 
 int64_t sort32(pic_ctx *c) {

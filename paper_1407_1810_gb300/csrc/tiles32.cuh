@@ -68,6 +68,21 @@ struct Args32 {
   float b0, r_min, omega_t;
 };
 
+// the particles [b0, b1) of a work unit (tile << 32 | index in the tile): its
+// even share of the tile's bin
+__device__ __forceinline__ void unit_range(const Args32 &A, long long u, int &tile, int64_t &b0, int64_t &b1) {
+  tile = (int)(u >> 32);
+  const int64_t s = A.start[(int64_t)tile * A.tc], n = A.start[(int64_t)(tile + 1) * A.tc] - s;
+  const int64_t m = (n + A.unit - 1) / A.unit, q = u & 0xffffffffll;
+  if (n < (1ll << 31) / 4096 && m < 4096) {  // 32-bit quotients
+    b0 = s + (int64_t)((uint32_t)n * (uint32_t)q / (uint32_t)m);
+    b1 = s + (int64_t)((uint32_t)n * (uint32_t)(q + 1) / (uint32_t)m);
+  } else {
+    b0 = s + n * q / m;
+    b1 = s + n * (q + 1) / m;
+  }
+}
+
 __device__ inline size_t pidx(const Args32 &A, int i, int j) {
   return (size_t)(i + A.PI) * (size_t)A.LD + (size_t)(j + A.PJ);
 }

@@ -788,10 +788,9 @@ __device__ __forceinline__ void tiles32_block(const Args32 &A, const Parts32 &P,
   int dead = 0;
   const float fs = __int_as_float((127 + KFIX - qexp_value(A.qexp)) << 23);  // 2^(KFIX - e)
   if (blk < (uint64_t)A.nunits) {
-    const long long u = A.units[blk];
-    const int t = (int)(u >> 32);
-    const int64_t b0 = A.start[(int64_t)t * A.tc] + (u & 0xffffffffll) * A.unit;
-    const int64_t b1 = min(A.start[(int64_t)(t + 1) * A.tc], b0 + A.unit);
+    int t;
+    int64_t b0, b1;
+    unit_range(A, A.units[blk], t, b0, b1);
     if (b1 <= b0) return;
     const int i0 = A.row0 + (t / A.ntj) * TI, j0 = (t % A.ntj) * TJ;
     const int wi0 = i0 - H - 1, wj0 = j0 - H - 1;
