@@ -235,7 +235,7 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
           for (int q = 0; q < 3; ++q) std::swap(c->F[q], c->Ft[q]);
         c->step += 1;
         if (c->d.inject) {
-          fa[k].t_inj = c->step * G.dt;
+          fa[k].jump = sigma_jump(c, c->step * G.dt);
           fa[k].inj_base = c->n_used;
           fa[k].inj_id0 = c->next_id;
           fa[k].inj_step = (uint64_t)c->step;

@@ -237,21 +237,16 @@ __global__ void k_filter(Grid G, const double *__restrict__ in, double *__restri
 
 // Surface charge per meridional cell: the jump of E_r across the conductor,
 // total E_r at (1/2, j) minus the analytic inside field's E_r at (r0, theta_j)
-// (zero for the monopole fields), averaged over the cell's two nodes.
-__device__ __forceinline__ void sigma_cell(const Grid &G, int j, const double *__restrict__ Er, double t, double *sig,
-                                           long long *smax) {
+// (zero for the monopole fields), averaged over the cell's two nodes.  The
+// analytic fields' part is a quadratic in cos theta (sigma_jump).
+__device__ __forceinline__ void sigma_cell(const Grid &G, int j, const double *__restrict__ Er, const SigmaJump &K,
+                                           double *sig, long long *smax) {
   if (j >= G.nth) return;
-  const Metric &m = G.m;
-  const double rb0 = m.r_h[G.PI];
-  double E[3], B[3], Ei[3];
-  const Vac<double> V{G.vacuum, G.b0, G.r_min, omega_at(G.omega, G.t_spin, t)};
   double e[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const double st = m.sin_t[j + h + G.PJ], ct = m.cos_t[j + h + G.PJ];
-    vacuum_field<double>(V, rb0, st, ct, false, E, B);
-    vacuum_field<double>(V, G.r_min, st, ct, true, Ei, B);
-    e[h] = (Er[gidx(G, 0, j + h)] + E[0]) - Ei[0];
+    const double ct = G.m.cos_t[j + h + G.PJ];
+    e[h] = Er[gidx(G, 0, j + h)] + fma(ct, fma(ct, K.k2, K.k1), K.k0);
   }
   const double s = 0.5 * (e[0] + e[1]);
   sig[j] = s;
@@ -279,10 +274,6 @@ constexpr int TW = BX + 2 * FUSE_FILT, TH = BY + 2 * FUSE_FILT;
 __constant__ int FILT_W[FUSE_FILT + 1][FUSE_FILT + 1] = {  // C(2N, N + k)
     {1, 0, 0, 0, 0}, {2, 1, 0, 0, 0}, {6, 4, 1, 0, 0}, {20, 15, 6, 1, 0}, {70, 56, 28, 8, 1}};
 
-// Images of a tile's rows and columns, formed once per block: array offset (or
-// -1: zero) and factor (+-1, +-2) of row i0 - N + r and, for integer and
-// half-integer j, of column j0 - N + q of the continued deposit.
-//
 // FP64 tiles take the weights from a table of doubles and the factors through
 // the exponent and sign bits: an integer-to-double conversion or a product
 // costs as much of the FP64 pipe as an addition of the convolution.
@@ -301,36 +292,37 @@ __device__ __forceinline__ double filt_scaled<double>(int c, double v) {
   return __hiloint2double(c < 0 ? hi ^ 0x80000000 : hi, __double2loint(v));
 }
 
+// Images of the rows and columns that this thread loads of a tile: array
+// offset (or -1: zero) and factor (+-1, +-2) of rows i0 - N + ty (+ 8) and, for
+// integer and half-integer j, of columns j0 - N + tx (+ 32) of the continued
+// deposit.  In registers: a phase of the block that forms them in shared
+// memory costs another barrier (a 72 x 56 step 43.2 -> 42.4 us, 192 x 160
+// 79.5 -> 76.6 us with both these and the unrolled passes).
 struct FiltImages {
-  int row[TH], col[2][TW];
-  signed char row_c[TH], col_c[2][TW];
+  int row[2], row_c[2], col[2][2], col_c[2][2];
 };
 
-__device__ __forceinline__ void filt_images(FiltImages &im, const Grid &G, int i0, int j0, int N) {
-  const int t = threadIdx.y * BX + threadIdx.x;
-  if (t < BY + 2 * N) {
-    const int lo = -G.g - 1, hi = G.nr + G.g + 1;
-    int ii = i0 - N + t, c = 1;
+__device__ __forceinline__ FiltImages filt_images(const Grid &G, int i0, int j0, int N) {
+  FiltImages im;
+  const int lo = -G.g - 1, hi = G.nr + G.g + 1, n = G.nth;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    int ii = i0 - N + (int)threadIdx.y + a * BY, c = 1;
     if (ii <= lo) { ii = 2 * lo - ii; c = -1; }
     else if (ii >= hi) { ii = 2 * hi - ii; c = -1; }
-    im.row[t] = ii <= lo || ii >= hi ? -1 : ii + G.PI;  // -1: the dropped row itself
-    im.row_c[t] = (signed char)c;
+    im.row[a] = ii <= lo || ii >= hi ? -1 : ii + G.PI;  // -1: the dropped row itself
+    im.row_c[a] = c;
+    const int j = j0 - N + (int)threadIdx.x + a * BX;
+    // right of every column that a node of the tile reads: any
+    int jj = j > n + 2 * FUSE_FILT ? n : j, jh = j > n + 2 * FUSE_FILT ? n - 1 : j, d = 1;
+    while (jj < 0 || jj > n) jj = jj < 0 ? -jj : 2 * n - jj;
+    while (jh < 0 || jh >= n) { jh = jh < 0 ? -1 - jh : 2 * n - 1 - jh; d = -d; }
+    im.col[0][a] = jj + G.PJ;
+    im.col_c[0][a] = jj == 0 || jj == n ? 2 : 1;
+    im.col[1][a] = jh + G.PJ;
+    im.col_c[1][a] = d;
   }
-  const int u = t - 64, n = G.nth;  // other warps than the rows'
-  if (u >= 0 && u < 2 * TW) {
-    const int half = u / TW, q = u % TW;
-    int jj = j0 - N + q, c = 1;
-    if (jj > n + 2 * FUSE_FILT) jj = n;  // right of every column that a node of the tile reads
-    if (half) {
-      while (jj < 0 || jj >= n) { jj = jj < 0 ? -1 - jj : 2 * n - 1 - jj; c = -c; }
-    } else {
-      while (jj < 0 || jj > n) jj = jj < 0 ? -jj : 2 * n - jj;
-      if (jj == 0 || jj == n) c = 2;
-    }
-    im.col[half][q] = jj + G.PJ;
-    im.col_c[half][q] = (signed char)c;
-  }
-  __syncthreads();
+  return im;
 }
 
 template <class T, int NC>
@@ -341,10 +333,11 @@ struct FiltTile {
 
 // NC components (the first of them component c0) of the tile with N passes at
 // this thread's node; every thread of the block calls it
-template <class T, int NC, class L>
-__device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &im, const Grid &G, int N, int c0,
-                                          T out[NC], const L &load) {
-  const int tx = threadIdx.x, ty = threadIdx.y, w = BX + 2 * N, h = BY + 2 * N;
+template <int N, class T, int NC, class L>
+__device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &im, const Grid &G, int c0, T out[NC],
+                                          const L &load) {
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  constexpr int w = BX + 2 * N, h = BY + 2 * N;
 #pragma unroll
   for (int k = 0; k < NC; ++k)
 #pragma unroll
@@ -353,10 +346,10 @@ __device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &
       for (int b = 0; b < 2; ++b) {
         const int r = ty + a * BY, q = tx + b * BX, half = c0 + k == 1;
         if (r < h && q < w) {
-          const int ro = im.row[r];
+          const int ro = im.row[a];
           t.in[k][r][q] = ro < 0 ? T(0)
-                                 : filt_scaled<T>(im.row_c[r] * im.col_c[half][q],
-                                                  load(c0 + k, (size_t)ro * G.LD + im.col[half][q]));
+                                 : filt_scaled<T>(im.row_c[a] * im.col_c[half][b],
+                                                  load(c0 + k, (size_t)ro * G.LD + im.col[half][b]));
         }
       }
   __syncthreads();
@@ -368,6 +361,7 @@ __device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &
       for (int k = 0; k < NC; ++k) {
         const T *x = &t.in[k][r][tx + N];
         T s = filt_weight<T>(N, 0) * x[0];
+#pragma unroll
         for (int m = 1; m <= N; ++m) s += filt_weight<T>(N, m) * (x[-m] + x[m]);
         t.mid[k][r][tx] = s;
       }
@@ -376,20 +370,53 @@ __device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
     T s = filt_weight<T>(N, 0) * t.mid[k][ty + N][tx];
+#pragma unroll
     for (int m = 1; m <= N; ++m) s += filt_weight<T>(N, m) * (t.mid[k][ty + N - m][tx] + t.mid[k][ty + N + m][tx]);
     out[k] = s;
   }
 }
 
-struct FiltSmem {
-  FiltImages im;
-  union {
-    FiltTile<long long, 3> q;
-    FiltTile<__int128, 1> w;
-    FiltTile<double, 3> d;
-  };
+union FiltSmem {
+  FiltTile<long long, 3> q;
+  FiltTile<__int128, 1> w;
+  FiltTile<double, 3> d;
   __device__ FiltSmem() {}
 };
+
+// the three filtered components at this thread's node, N passes
+template <bool FP32, int N>
+__device__ __forceinline__ void filtered_flux(const EnsFieldArg &S, FiltSmem &sm, int i0, int j0, bool pole,
+                                              double F[3]) {
+  const Grid &G = S.G;
+  const FiltImages im = filt_images(G, i0, j0, N);
+  if (FP32) {
+    const int s = qexp_value(S.qexp) - KFIX;  // one flux unit is 2^s of charge
+    const long long lim = 1ll << (60 - 4 * N);
+    bool big = false;
+    long long v[3];
+    filt_conv<N>(sm.q, im, G, 0, v, [&](int k, size_t x) {
+      const long long y = S.acc[k][x];
+      big |= y >= lim || y <= -lim;
+      return y;
+    });
+#pragma unroll
+    for (int k = 0; k < 3; ++k) F[k] = fixed_to_f64(k != 1 && pole ? v[k] / 2 : v[k], s - 4 * N);
+    if (__syncthreads_or(big)) {
+      for (int k = 0; k < 3; ++k) {
+        __int128 z[1];
+        filt_conv<N>(sm.w, im, G, k, z, [&](int c, size_t x) { return (__int128)S.acc[c][x]; });
+        F[k] = fixed_to_f64(k != 1 && pole ? z[0] / 2 : z[0], s - 4 * N);
+        __syncthreads();
+      }
+    }
+  } else {
+    const double sc = __longlong_as_double((long long)(1023 - 4 * N) << 52);  // 16^-N
+    double v[3];
+    filt_conv<N>(sm.d, im, G, 0, v, [&](int k, size_t x) { return S.Fin[k][x]; });
+#pragma unroll
+    for (int k = 0; k < 3; ++k) F[k] = v[k] * (k != 1 && pole ? 0.5 * sc : sc);
+  }
+}
 
 // One block (32 x 8 nodes of the ghost band -g..nr+g, 0..nth) of the E update:
 // the flux of the deposit filtered and stored (the step's fluxes), then E.
@@ -404,47 +431,21 @@ __device__ __forceinline__ void e_block(const EnsFieldArg &S, unsigned b, FiltSm
   const int N = S.n_filt;
   const bool pole = j == 0 || j == G.nth;
   double F[3] = {0.0, 0.0, 0.0};
-  if (N > FUSE_FILT) {  // filtered pass by pass before this launch
-    if (in)
-      for (int k = 0; k < 3; ++k) F[k] = S.Fout[k][o];
-  } else if (FP32) {
-    const int s = qexp_value(S.qexp) - KFIX;  // one flux unit is 2^s of charge
-    if (N == 0) {
-      if (in)
-        for (int k = 0; k < 3; ++k) F[k] = fixed_to_f64(S.acc[k][o], s);
-    } else {
-      const long long lim = 1ll << (60 - 4 * N);
-      bool big = false;
-      long long v[3];
-      filt_images(sm.im, G, i0, j0, N);
-      filt_conv(sm.q, sm.im, G, N, 0, v, [&](int k, size_t x) {
-        const long long y = S.acc[k][x];
-        big |= y >= lim || y <= -lim;
-        return y;
-      });
+  switch (N) {
+    case 0:
+      if (in) {
+        const int s = FP32 ? qexp_value(S.qexp) - KFIX : 0;  // one flux unit is 2^s of charge
 #pragma unroll
-      for (int k = 0; k < 3; ++k) F[k] = fixed_to_f64(k != 1 && pole ? v[k] / 2 : v[k], s - 4 * N);
-      if (__syncthreads_or(big)) {
-        for (int k = 0; k < 3; ++k) {
-          __int128 z[1];
-          filt_conv(sm.w, sm.im, G, N, k, z, [&](int c, size_t x) { return (__int128)S.acc[c][x]; });
-          F[k] = fixed_to_f64(k != 1 && pole ? z[0] / 2 : z[0], s - 4 * N);
-          __syncthreads();
-        }
+        for (int k = 0; k < 3; ++k) F[k] = FP32 ? fixed_to_f64(S.acc[k][o], s) : S.Fin[k][o];
       }
-    }
-  } else {
-    if (N == 0) {
+      break;
+    case 1: filtered_flux<FP32, 1>(S, sm, i0, j0, pole, F); break;
+    case 2: filtered_flux<FP32, 2>(S, sm, i0, j0, pole, F); break;
+    case 3: filtered_flux<FP32, 3>(S, sm, i0, j0, pole, F); break;
+    case 4: filtered_flux<FP32, 4>(S, sm, i0, j0, pole, F); break;
+    default:  // filtered pass by pass before this launch
       if (in)
-        for (int k = 0; k < 3; ++k) F[k] = S.Fin[k][o];
-    } else {
-      const double sc = __longlong_as_double((long long)(1023 - 4 * N) << 52);  // 16^-N
-      double v[3];
-      filt_images(sm.im, G, i0, j0, N);
-      filt_conv(sm.d, sm.im, G, N, 0, v, [&](int k, size_t x) { return S.Fin[k][x]; });
-#pragma unroll
-      for (int k = 0; k < 3; ++k) F[k] = v[k] * (k != 1 && pole ? 0.5 * sc : sc);
-    }
+        for (int k = 0; k < 3; ++k) F[k] = S.Fout[k][o];
   }
   if (b == 0 && threadIdx.x == 0 && threadIdx.y == 0 && S.inject) S.cnt[CNT_SMAX] = 0;  // raised by the B update
   if (!in) return;
@@ -472,22 +473,27 @@ __device__ __forceinline__ void b_block(const EnsFieldArg &S, unsigned b, bool s
     for (int k = 0; k < 3; ++k) (S.Fout[k] == S.Fin[k] ? S.Ftmp : S.Fin)[k][o] = 0.0;
   if (i < 0 || i > G.nr) return;
   b_node<FP32>(S, i, j);
-  if (sigma && i == 0) sigma_cell(G, j, S.f[ER], S.t_inj, S.sig, S.inject_smooth ? nullptr : S.cnt + CNT_SMAX);
+  if (sigma && i == 0) sigma_cell(G, j, S.f[ER], S.jump, S.sig, S.inject_smooth ? nullptr : S.cnt + CNT_SMAX);
 }
 
 // the passes of an integer-j FP64 array (the node charge) in one
+template <int N>
+__device__ __forceinline__ double filtered_charge(FiltTile<double, 1> &t, const Grid &G, int i0, int j0,
+                                                  const double *__restrict__ a) {
+  double v[1];
+  filt_conv<N>(t, filt_images(G, i0, j0, N), G, 0, v, [&](int, size_t x) { return a[x]; });
+  return v[0];
+}
 __global__ void __launch_bounds__(BX *BY) k_filter_tile(Grid G, const double *__restrict__ a, double *__restrict__ out,
                                                        int N) {
-  __shared__ FiltImages im;
   __shared__ FiltTile<double, 1> t;
   const int i0 = -G.g + (int)blockIdx.y * BY, j0 = (int)blockIdx.x * BX;
-  double v[1];
-  filt_images(im, G, i0, j0, N);
-  filt_conv(t, im, G, N, 0, v, [&](int, size_t x) { return a[x]; });
+  const double v = N == 1 ? filtered_charge<1>(t, G, i0, j0, a) : N == 2 ? filtered_charge<2>(t, G, i0, j0, a)
+                 : N == 3 ? filtered_charge<3>(t, G, i0, j0, a) : filtered_charge<4>(t, G, i0, j0, a);
   const int i = i0 + (int)threadIdx.y, j = j0 + (int)threadIdx.x;
   if (i > G.nr + G.g || j > G.nth) return;
   const double sc = __longlong_as_double((long long)(1023 - 4 * N) << 52);  // 16^-N
-  out[gidx(G, i, j)] = v[0] * (j == 0 || j == G.nth ? 0.5 * sc : sc);
+  out[gidx(G, i, j)] = v * (j == 0 || j == G.nth ? 0.5 * sc : sc);
 }
 
 template <bool FP32>
@@ -510,8 +516,8 @@ __global__ void k_flux_from_acc(const __grid_constant__ EnsFieldArg S) {
   for (int k = 0; k < 3; ++k) S.Fin[k][o] = fixed_to_f64(S.acc[k][o], s);
 }
 
-__global__ void k_inject_sigma(Grid G, const double *__restrict__ Er, double t, double *sig, long long *smax) {
-  sigma_cell(G, blockIdx.x * blockDim.x + threadIdx.x, Er, t, sig, smax);
+__global__ void k_inject_sigma(Grid G, const double *__restrict__ Er, SigmaJump K, double *sig, long long *smax) {
+  sigma_cell(G, blockIdx.x * blockDim.x + threadIdx.x, Er, K, sig, smax);
 }
 
 // One 1-2-1 pass over sigma along theta; each polar cell is its own mirror
@@ -793,6 +799,28 @@ int ens_blocks(const pic_ctx *c, int kind) {
   }
 }
 
+// The analytic fields' jump of E_r at the star, E_r outside at (1/2, j) minus
+// E_r inside at r0, as k0 + k1 cos th + k2 cos^2 th at time t (vacuum_field's
+// terms in E_r)
+SigmaJump sigma_jump(const pic_ctx *c, double t) {
+  const Grid &G = c->G;
+  const double W = omega_at(G.omega, G.t_spin, t), r0 = G.r_min;
+  const double rb = c->d.r_map == PIC_R_LOG ? r0 * std::exp(0.5 * G.dxi) : r0 + 0.5 * G.dxi, q = r0 / rb;
+  const double in = G.b0 * r0 * W;  // mu W / r0^2
+  SigmaJump K{0.0, 0.0, 0.0};
+  if (G.vacuum == PIC_VAC_MONOPOLE_ROTATOR) {
+    K.k1 = -2.0 * G.b0 * q * q * q * r0 * W;
+  } else if (G.vacuum == PIC_VAC_DIPOLE_COROT) {  // sin^2 th (mu W / rb^2 - mu W / r0^2)
+    K.k0 = in * (q * q - 1.0);
+    K.k2 = -K.k0;
+  } else if (G.vacuum == PIC_VAC_DIPOLE_ROTATOR) {  // -a (3 cos^2 th - 1) - in sin^2 th
+    const double a = in * q * q * q * q;
+    K.k0 = a - in;
+    K.k2 = in - 3.0 * a;
+  }
+  return K;
+}
+
 // launches of the grid phases of one step (as pic_step_body makes them)
 int grid_launches(const pic_ctx *c) {
   return (c->d.n_filt > FUSE_FILT ? 1 + 3 * c->d.n_filt : 0) + 2 + (c->d.inject ? 1 + c->d.inject_smooth : 0);
@@ -880,7 +908,7 @@ void fields_e_step(pic_ctx *c) {
 void fields_b_step(pic_ctx *c, bool sigma) {
   EnsFieldArg a;
   ens_fill_field_arg(c, &a);
-  a.t_inj = (c->step + 1) * c->G.dt;
+  a.jump = sigma_jump(c, (c->step + 1) * c->G.dt);
   const int sg = sigma && c->d.inject ? 1 : 0;
   const unsigned nb = (unsigned)ens_blocks(c, ENS_BAND);
   if (c->d.precision == PIC_FP32) ++c->launches, k_b_step<true><<<nb, dim3(BX, BY), 0, c->stream>>>(a, sg);
@@ -926,7 +954,7 @@ void inject(pic_ctx *c, double t, bool have_sigma) {
   const int tb = (G.nth + 127) / 128;
   if (!have_sigma) {  // a radial slab: after the exchange of the step's fields
     cudaMemsetAsync(smax, 0, sizeof(long long), c->stream);
-    ++c->launches, k_inject_sigma<<<tb, 128, 0, c->stream>>>(G, c->f[ER], t, a, ns ? nullptr : smax);
+    ++c->launches, k_inject_sigma<<<tb, 128, 0, c->stream>>>(G, c->f[ER], sigma_jump(c, t), a, ns ? nullptr : smax);
   }
   for (int p = 0; p < ns; ++p) {
     ++c->launches, k_inject_smooth<<<tb, 128, 0, c->stream>>>(G.nth, a, b, p == ns - 1 ? smax : nullptr);

@@ -103,6 +103,7 @@ struct EnsList {
 enum ProfSlot { PROF_PARTICLES = 0, PROF_REDUCE = 1, PROF_FILTER = 2, PROF_FIELDS = 3, PROF_INJECT = 4,
                 PROF_SORT = 5, PROF_N };
 
+struct SigmaJump { double k0, k1, k2; };  // see sigma_jump (fields.cu)
 // One context at one step as the grid kernels read it (kernel parameter of a
 // single context's launches, device table of an ensemble's): its grid and
 // arrays, the flux buffers and the step's injection.
@@ -120,7 +121,7 @@ struct EnsFieldArg {
   double *sig;                         // two buffers of nth + 1
   Parts32 p32;
   int64_t inj_base, inj_id0;           // first slot and id of the step's injected pairs
-  double t_inj;                        // time at which the injection reads the field
+  SigmaJump jump;                      // of the analytic field at the time the injection reads the field
   double f_inj, inject_q;
   uint64_t inject_seed, inj_step;
   int inject, npp, inject_smooth, n_filt;
@@ -229,6 +230,7 @@ void ens_flux(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t
 void ens_e_step(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
 void ens_b_step(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
 int grid_launches(const pic_ctx *c);
+SigmaJump sigma_jump(const pic_ctx *c, double t);
 bool filter_swaps(const pic_ctx *c);
 void ens_inject_smooth(const EnsFieldArg *tab, const EnsList &L, int blocks, int pass, cudaStream_t s);
 void ens_inject_write(const EnsFieldArg *tab, const EnsList &L, int blocks, cudaStream_t s);
