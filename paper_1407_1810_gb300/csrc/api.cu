@@ -822,10 +822,23 @@ int pic_prepare_steps(pic_ctx *c, int steps) {
   return PIC_OK;
 }
 
+// Overlapped launches for the length of a scope, unless the stream is being
+// captured (a graph's kernel nodes keep their full dependencies).
+struct Overlap {
+  pic_ctx *c;
+  explicit Overlap(pic_ctx *ctx) : c(ctx) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+    else c->overlap = st == cudaStreamCaptureStatusNone;
+  }
+  ~Overlap() { c->overlap = false; }
+};
+
 extern "C" int pic_step(pic_ctx *c, int32_t nsteps) {
   if (!c) return pic_fail(PIC_EINVAL, "null context");
   if (nsteps < 0) return pic_fail(PIC_EINVAL, "nsteps < 0");
   int done = 0;
+  const Overlap overlap(c);
   while (done < nsteps) {
     // steps up to the next sort run without host synchronisation
     int block = std::min(nsteps - done, std::max(1, c->d.sort_interval - c->steps_since_sort));

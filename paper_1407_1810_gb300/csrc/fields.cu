@@ -232,6 +232,7 @@ __device__ __forceinline__ void filter_node(const Grid &G, int i, int j, const d
 }
 
 __global__ void k_filter(Grid G, const double *__restrict__ in, double *__restrict__ out, int half_j) {
+  follow();
   filter_node(G, -G.g + (int)(blockIdx.y * BY + threadIdx.y), blockIdx.x * BX + threadIdx.x, in, out, half_j);
 }
 
@@ -499,15 +500,18 @@ __global__ void __launch_bounds__(BX *BY) k_filter_tile(Grid G, const double *__
 template <bool FP32>
 __global__ void __launch_bounds__(BX *BY) k_e_step(const __grid_constant__ EnsFieldArg S) {
   __shared__ FiltSmem sm;
+  follow();
   e_block<FP32>(S, blockIdx.x, sm);
 }
 template <bool FP32>
 __global__ void __launch_bounds__(BX *BY) k_b_step(const __grid_constant__ EnsFieldArg S, int sigma) {
+  follow();
   b_block<FP32>(S, blockIdx.x, sigma != 0);
 }
 
 // fixed point -> FP64 fluxes over the ghost band, for the pass-by-pass filter
 __global__ void k_flux_from_acc(const __grid_constant__ EnsFieldArg S) {
+  follow();
   const Grid &G = S.G;
   const int i = -G.g + (int)(blockIdx.y * BY + threadIdx.y), j = blockIdx.x * BX + threadIdx.x;
   if (i > G.nr + G.g || j > G.nth) return;
@@ -532,6 +536,7 @@ __device__ __forceinline__ void smooth_cell(int j, int nth, const double *__rest
 }
 
 __global__ void k_inject_smooth(int nth, const double *__restrict__ in, double *out, long long *smax) {
+  follow();
   smooth_cell(blockIdx.x * blockDim.x + threadIdx.x, nth, in, out, smax);
 }
 
@@ -622,6 +627,7 @@ template <bool FP32>
 __global__ void k_inject_write(Grid G, const double *__restrict__ sig, const long long *smax, Parts64 P,
                                Parts32 Q, int64_t base, int64_t id0, InjectRule R, long long *cnt,
                                long long *capped_cnt, long long *qexp) {
+  follow();
   inject_slot<FP32>(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, G, sig, smax, P, Q, base, id0, R, cnt,
                     capped_cnt, qexp);
 }
@@ -894,15 +900,15 @@ void fields_e_step(pic_ctx *c) {
   if (c->d.n_filt > FUSE_FILT) {
     const Grid &G = c->G;
     const dim3 gr = grid2(G.nr + 2 * G.g + 1, G.nth + 1);
-    if (fp32) ++c->launches, k_flux_from_acc<<<gr, dim3(BX, BY), 0, c->stream>>>(a);
+    if (fp32) ++c->launches, launch_on(c->stream, c->overlap, k_flux_from_acc, gr, dim3(BX, BY), a);
     for (int p = 0; p < c->d.n_filt; ++p)
       for (int k = 0; k < 3; ++k)
-        ++c->launches, k_filter<<<gr, dim3(BX, BY), 0, c->stream>>>(G, (p & 1) ? a.Ftmp[k] : a.Fin[k],
+        ++c->launches, launch_on(c->stream, c->overlap, k_filter, gr, dim3(BX, BY), G, (p & 1) ? a.Ftmp[k] : a.Fin[k],
                                                                     (p & 1) ? a.Fin[k] : a.Ftmp[k], k == 1);
   }
   const unsigned nb = (unsigned)ens_blocks(c, ENS_BAND);
-  if (fp32) ++c->launches, k_e_step<true><<<nb, dim3(BX, BY), 0, c->stream>>>(a);
-  else ++c->launches, k_e_step<false><<<nb, dim3(BX, BY), 0, c->stream>>>(a);
+  if (fp32) ++c->launches, launch_on(c->stream, c->overlap, k_e_step<true>, nb, dim3(BX, BY), a);
+  else ++c->launches, launch_on(c->stream, c->overlap, k_e_step<false>, nb, dim3(BX, BY), a);
 }
 
 void fields_b_step(pic_ctx *c, bool sigma) {
@@ -911,8 +917,8 @@ void fields_b_step(pic_ctx *c, bool sigma) {
   a.jump = sigma_jump(c, (c->step + 1) * c->G.dt);
   const int sg = sigma && c->d.inject ? 1 : 0;
   const unsigned nb = (unsigned)ens_blocks(c, ENS_BAND);
-  if (c->d.precision == PIC_FP32) ++c->launches, k_b_step<true><<<nb, dim3(BX, BY), 0, c->stream>>>(a, sg);
-  else ++c->launches, k_b_step<false><<<nb, dim3(BX, BY), 0, c->stream>>>(a, sg);
+  if (c->d.precision == PIC_FP32) ++c->launches, launch_on(c->stream, c->overlap, k_b_step<true>, nb, dim3(BX, BY), a, sg);
+  else ++c->launches, launch_on(c->stream, c->overlap, k_b_step<false>, nb, dim3(BX, BY), a, sg);
   // the filtered flux stays in F (pic_get_flux), the cleared deposit in Ft
   if (a.Fout[0] != c->F[0])
     for (int k = 0; k < 3; ++k) std::swap(c->F[k], c->Ft[k]);
@@ -957,17 +963,17 @@ void inject(pic_ctx *c, double t, bool have_sigma) {
     ++c->launches, k_inject_sigma<<<tb, 128, 0, c->stream>>>(G, c->f[ER], sigma_jump(c, t), a, ns ? nullptr : smax);
   }
   for (int p = 0; p < ns; ++p) {
-    ++c->launches, k_inject_smooth<<<tb, 128, 0, c->stream>>>(G.nth, a, b, p == ns - 1 ? smax : nullptr);
+    ++c->launches, launch_on(c->stream, c->overlap, k_inject_smooth, tb, 128, G.nth, a, b, p == ns - 1 ? smax : nullptr);
     double *x = a; a = b; b = x;
   }
   const InjectRule R{c->d.inject, npp, c->d.f_inj, c->d.inject_q, c->d.inject_seed, (uint64_t)c->step};
   const int64_t nslots = (int64_t)G.nth * npp * 2;
   const int blocks = (int)((nslots + 255) / 256);
   if (c->d.precision == PIC_FP32)
-    ++c->launches, k_inject_write<true><<<blocks, 256, 0, c->stream>>>(G, a, smax, c->p64, c->p32, c->n_used, c->next_id, R,
+    ++c->launches, launch_on(c->stream, c->overlap, k_inject_write<true>, blocks, 256, G, a, smax, c->p64, c->p32, c->n_used, c->next_id, R,
                                                         c->d_cnt + CNT_INJECTED, c->d_cnt + CNT_CAPPED, c->qexp);
   else
-    ++c->launches, k_inject_write<false><<<blocks, 256, 0, c->stream>>>(G, a, smax, c->p64, c->p32, c->n_used, c->next_id, R,
+    ++c->launches, launch_on(c->stream, c->overlap, k_inject_write<false>, blocks, 256, G, a, smax, c->p64, c->p32, c->n_used, c->next_id, R,
                                                          c->d_cnt + CNT_INJECTED, c->d_cnt + CNT_CAPPED, c->qexp);
   c->n_used += nslots;
   c->next_id += nslots;

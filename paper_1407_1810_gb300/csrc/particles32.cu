@@ -102,7 +102,10 @@ __device__ __forceinline__ void scan_bins_block(int64_t *count, int64_t *start, 
   if (t == 1023) start[nb] = part[1023];
 }
 
-__global__ void k_scan_bins(int64_t *count, int64_t *start, int nb) { scan_bins_block(count, start, nb); }
+__global__ void k_scan_bins(int64_t *count, int64_t *start, int nb) {
+  follow();
+  scan_bins_block(count, start, nb);
+}
 
 // block sum of 256 values (all threads get it)
 __device__ inline int64_t block_sum256(int64_t v, int64_t *sm) {
@@ -129,6 +132,7 @@ __device__ __forceinline__ void scan_sums_block(const int64_t *count, int64_t nb
 }
 
 __global__ void k_scan_sums(const int64_t *count, int64_t nb, int64_t *sums) {
+  follow();
   scan_sums_block(count, nb, sums, blockIdx.x);
 }
 
@@ -160,6 +164,7 @@ __device__ __forceinline__ void scan_apply_block(int64_t *count, int64_t *start,
 }
 
 __global__ void k_scan_apply(int64_t *count, int64_t *start, int64_t nb, const int64_t *offs, int nblk) {
+  follow();
   scan_apply_block(count, start, nb, offs, nblk, blockIdx.x);
 }
 
@@ -172,6 +177,7 @@ __device__ __forceinline__ void unit_count_at(int t, const int64_t *start, int t
 }
 
 __global__ void k_unit_count(const int64_t *start, int tc, int ntiles, int64_t unit, int64_t *ucount) {
+  follow();
   unit_count_at(blockIdx.x * blockDim.x + threadIdx.x, start, tc, ntiles, unit, ucount);
 }
 
@@ -182,6 +188,7 @@ __device__ __forceinline__ void unit_fill_at(int t, const int64_t *uoff, int nti
 }
 
 __global__ void k_unit_fill(const int64_t *uoff, int ntiles, long long *units) {
+  follow();
   unit_fill_at(blockIdx.x * blockDim.x + threadIdx.x, uoff, ntiles, units);
 }
 
@@ -232,6 +239,7 @@ __device__ __forceinline__ void scatter_block(const Args32 &A, const Parts32 &S,
 }
 
 __global__ void k_scatter_cells(Args32 A, Parts32 S, Parts32 D, int64_t n, int64_t *cursor) {
+  follow();
   scatter_block(A, S, D, n, cursor, blockIdx.x);
 }
 
@@ -609,7 +617,7 @@ void particles32(pic_ctx *c, double t) {
   const TileMaps &M = *reinterpret_cast<const TileMaps *>(c->tile_maps[c->d.tile_shape]);
   const int shape = c->tiles.TI == 8 ? 1 : (c->tiles.TI == 32 ? 2 : 0);
   ++c->launches;
-  (use_packed(c) ? launch_two : launch_one)(tile_spec(c), shape, (unsigned)blocks, c->stream, A, c->p32, M);
+  (use_packed(c) ? launch_two : launch_one)(tile_spec(c), shape, (unsigned)blocks, c->stream, c->overlap, A, c->p32, M);
 }
 
 }  // namespace pic
@@ -749,18 +757,18 @@ int64_t sort32(pic_ctx *c) {
   const unsigned blocks = (unsigned)((n + 255) / 256);
   const int nblk = (int)((T.nbins + SCAN_CHUNK - 1) / SCAN_CHUNK);
   ++c->launches, k_hist<<<blocks, 256, 0, c->stream>>>(A, c->p32, n, count);
-  ++c->launches, k_scan_sums<<<nblk, 256, 0, c->stream>>>(count, T.nbins, T.bsum);
-  ++c->launches, k_scan_bins<<<1, 1024, 0, c->stream>>>(T.bsum, T.bsum + nblk + 1, nblk);
-  ++c->launches, k_scan_apply<<<nblk, 256, 0, c->stream>>>(count, T.start, T.nbins, T.bsum + nblk + 1, nblk);
-  ++c->launches, k_scatter_cells<<<blocks, 256, 0, c->stream>>>(A, c->p32, c->q32, n, count);
+  ++c->launches, launch_on(c->stream, c->overlap, k_scan_sums, nblk, 256, count, T.nbins, T.bsum);
+  ++c->launches, launch_on(c->stream, c->overlap, k_scan_bins, 1, 1024, T.bsum, T.bsum + nblk + 1, nblk);
+  ++c->launches, launch_on(c->stream, c->overlap, k_scan_apply, nblk, 256, count, T.start, T.nbins, T.bsum + nblk + 1, nblk);
+  ++c->launches, launch_on(c->stream, c->overlap, k_scatter_cells, blocks, 256, A, c->p32, c->q32, n, count);
   // the work units of the tile kernel (n bounds the live count from above)
   const unsigned tb = (unsigned)((T.ntiles + 255) / 256);
   const int ublk = (int)((T.ntiles + SCAN_CHUNK - 1) / SCAN_CHUNK);
-  ++c->launches, k_unit_count<<<tb, 256, 0, c->stream>>>(T.start, T.tc, T.ntiles, T.unit, T.ucount);
-  ++c->launches, k_scan_sums<<<ublk, 256, 0, c->stream>>>(T.ucount, T.ntiles, T.usum);
-  ++c->launches, k_scan_bins<<<1, 1024, 0, c->stream>>>(T.usum, T.usum + ublk + 1, ublk);
-  ++c->launches, k_scan_apply<<<ublk, 256, 0, c->stream>>>(T.ucount, T.ucount, T.ntiles, T.usum + ublk + 1, ublk);
-  ++c->launches, k_unit_fill<<<tb, 256, 0, c->stream>>>(T.ucount, T.ntiles, T.units);
+  ++c->launches, launch_on(c->stream, c->overlap, k_unit_count, tb, 256, T.start, T.tc, T.ntiles, T.unit, T.ucount);
+  ++c->launches, launch_on(c->stream, c->overlap, k_scan_sums, ublk, 256, T.ucount, T.ntiles, T.usum);
+  ++c->launches, launch_on(c->stream, c->overlap, k_scan_bins, 1, 1024, T.usum, T.usum + ublk + 1, ublk);
+  ++c->launches, launch_on(c->stream, c->overlap, k_scan_apply, ublk, 256, T.ucount, T.ucount, T.ntiles, T.usum + ublk + 1, ublk);
+  ++c->launches, launch_on(c->stream, c->overlap, k_unit_fill, tb, 256, T.ucount, T.ntiles, T.units);
   // particles in cell bins: everything before the bin of removed ones; units
   cudaMemcpyAsync(c->h_pinned, T.start + (int64_t)T.ntiles * T.tc, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream);
   cudaMemcpyAsync(c->h_pinned + 1, T.ucount + T.ntiles, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream);

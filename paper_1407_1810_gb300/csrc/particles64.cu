@@ -235,6 +235,7 @@ struct Args64 {
 
 __global__ void __launch_bounds__(256) k_particles64(const __grid_constant__ Args64 A, Parts64 P, int64_t n,
                                                      Fields64 F, Flux64 D, int *err, long long *cnt, AxisTies ties) {
+  follow();
   const Grid &G = A.G;
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (k >= n) return;
@@ -496,8 +497,8 @@ void particles64(pic_ctx *c, double t) {
   A.series_t = G.nth >= 32;
   A.th_n = c->th_n64;
   const int64_t blocks = (c->n_used + 255) / 256;
-  ++c->launches, k_particles64<<<(unsigned)blocks, 256, 0, c->stream>>>(A, c->p64, c->n_used, F, D, c->d_err, c->d_cnt,
-                                                                          axis_ties(c));
+  ++c->launches, launch_on(c->stream, c->overlap, k_particles64, (unsigned)blocks, 256, A, c->p64, c->n_used, F, D,
+                           c->d_err, c->d_cnt, axis_ties(c));
 }
 
 int64_t compact64(pic_ctx *c) {

@@ -136,6 +136,7 @@ enum EnsKind { ENS_FLUX = 0, ENS_FILTER, ENS_BAND, ENS_SMOOTH, ENS_WRITE, ENS_NK
 struct pic_ctx {
   pic_desc d{};
   cudaStream_t stream = nullptr;
+  bool overlap = false;  // inside pic_step, not under capture: kernels launched as dependents (launch_on)
   int device = 0;
   pic::Grid G{};
   void *block = nullptr;        // the allocation that holds the context's own arrays

@@ -185,9 +185,9 @@ static_assert(sizeof(EnsTileBatch) <= 32000, "kernel parameters are limited to 3
 
 // launches a form's tile kernel: the shape (0: 16 x 16, 1: 8 x 32, 2: 32 x 8)
 // and specialisation of one context, or of the members of a batch
-void launch_one(int spec, int shape, unsigned blocks, cudaStream_t s, const Args32 &A, const Parts32 &P,
+void launch_one(int spec, int shape, unsigned blocks, cudaStream_t s, bool overlap, const Args32 &A, const Parts32 &P,
                 const TileMaps &M);
-void launch_two(int spec, int shape, unsigned blocks, cudaStream_t s, const Args32 &A, const Parts32 &P,
+void launch_two(int spec, int shape, unsigned blocks, cudaStream_t s, bool overlap, const Args32 &A, const Parts32 &P,
                 const TileMaps &M);
 void launch_ens_one(int spec, int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &B);
 void launch_ens_two(int spec, int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &B);

@@ -552,6 +552,7 @@ __device__ __forceinline__ void tiles32_block(const Args32 &A, const Parts32 &P,
 
 template <int TI, int TJ, int SPEC>
 __global__ void __launch_bounds__(NT, 4) k_tiles32(Args32 A, Parts32 P, const __grid_constant__ TileMaps maps) {
+  follow();
   tiles32_block<TI, TJ, SPEC, false>(A, P, maps.m, blockIdx.x);
 }
 
@@ -569,10 +570,10 @@ __global__ void __launch_bounds__(NT, 4) k_ens_tiles32(const __grid_constant__ E
 }
 
 template <int SPEC>
-void launch(int shape, unsigned blocks, cudaStream_t s, const Args32 &A, const Parts32 &P, const TileMaps &M) {
-  if (shape == 1) k_tiles32<8, 32, SPEC><<<blocks, NT, 0, s>>>(A, P, M);
-  else if (shape == 2) k_tiles32<32, 8, SPEC><<<blocks, NT, 0, s>>>(A, P, M);
-  else k_tiles32<16, 16, SPEC><<<blocks, NT, 0, s>>>(A, P, M);
+void launch(int shape, unsigned blocks, cudaStream_t s, bool overlap, const Args32 &A, const Parts32 &P, const TileMaps &M) {
+  if (shape == 1) launch_on(s, overlap, k_tiles32<8, 32, SPEC>, blocks, NT, A, P, M);
+  else if (shape == 2) launch_on(s, overlap, k_tiles32<32, 8, SPEC>, blocks, NT, A, P, M);
+  else launch_on(s, overlap, k_tiles32<16, 16, SPEC>, blocks, NT, A, P, M);
 }
 
 template <int SPEC>
@@ -584,11 +585,11 @@ void launch_ens(int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &
 
 }  // namespace
 
-void launch_one(int spec, int shape, unsigned blocks, cudaStream_t s, const Args32 &A, const Parts32 &P,
+void launch_one(int spec, int shape, unsigned blocks, cudaStream_t s, bool overlap, const Args32 &A, const Parts32 &P,
                 const TileMaps &M) {
-  if (spec == SPEC_MONOPOLE) launch<SPEC_MONOPOLE>(shape, blocks, s, A, P, M);
-  else if (spec == SPEC_ROTATOR) launch<SPEC_ROTATOR>(shape, blocks, s, A, P, M);
-  else launch<SPEC_GENERIC>(shape, blocks, s, A, P, M);
+  if (spec == SPEC_MONOPOLE) launch<SPEC_MONOPOLE>(shape, blocks, s, overlap, A, P, M);
+  else if (spec == SPEC_ROTATOR) launch<SPEC_ROTATOR>(shape, blocks, s, overlap, A, P, M);
+  else launch<SPEC_GENERIC>(shape, blocks, s, overlap, A, P, M);
 }
 
 void launch_ens_one(int spec, int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &B) {
