@@ -20,7 +20,9 @@ namespace {
 // approximations; compares are made on the integer halves of a double.
 // Measured on 512 x 512, 2e7 particles: 634 FP64 instructions a particle and
 // 22.6 ms a step with exp, log, sincos, atan2, hypot and divisions in global
-// coordinates; 300 and 11.2 ms so (the FP64 pipe at its 86 % limit in both).
+// coordinates; 300 and 11.2 ms so; 10.7 ms with FP32 last terms of the series
+// and one code for the last path segment of crossing and other lanes (the FP64
+// pipe at its 86 % limit throughout).
 // The local form is also the more exact one: against 50 digits, a move's
 // position error falls from 1.2e-14 to 3.5e-15 cell, and next to a pole (1e-6
 // to 1 cell from it) the momenta's from 1e-10 to 2e-15.
@@ -48,21 +50,40 @@ __device__ __forceinline__ double rsqrt64(double x) {
   return (unsigned)hi_word(x) - 0x00100000u < 0x7fe00000u ? r : y;  // normal, positive, finite x
 }
 
-// sqrt(x) with one Newton correction of x rsqrt(x)
+// sqrt(x) = g + d y (1 / 2 + 3 d y^2 / 8), g = x y with y the approximation of
+// 1 / sqrt(x), d = x - g^2 exact: the rounding of g does not stay in the result
 __device__ __forceinline__ double sqrt64(double x) {
-  const double y = rsqrt64(x), g = x * y;
-  const double r = fma(0.5 * y, fma(-g, g, x), g);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double g = x * y, t = fma(-g, g, x) * y;
+  const double r = fma(t, fma(0.375, t * y, 0.5), g);
   return (unsigned)hi_word(x) - 0x00100000u < 0x7fe00000u ? r : sqrt(x);
 }
 
+// The last terms of a series, too small for their 24 bits to show in a double,
+// are summed in FP32; the arguments are converted with integer operations
+// (toward zero; a subnormal float becomes 0), as a conversion instruction
+// costs as much of the FP64 pipe as a term.
+__device__ __forceinline__ float low32(double x) {  // |x| < 2
+  const int e = (hi_word(x) & 0x7fffffff) - 0x38000000;
+  const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)(e < 0x00100000 ? 0 : e), 3));
+  return hi_word(x) < 0 ? -f : f;
+}
+__device__ __forceinline__ double high64(float x) {  // normal, positive x
+  const unsigned b = __float_as_uint(x);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
 // arcsine for |t| < 1/8: t sum (2k)! / (4^k k!^2 (2k+1)) t^2k, truncated below
-// 2^-60 relative
+// 2^-60 relative; FP32 from t^10 on (2^-35 of t)
 __device__ __forceinline__ double asin_series64(double t) {
   const double z = t * t;
-  double p = 6435.0 / 557056.0;
-  p = fma(p, z, 143.0 / 10240.0);
-  p = fma(p, z, 231.0 / 13312.0);
-  p = fma(p, z, 63.0 / 2816.0);
+  const float y = low32(z);
+  float q = 6435.0f / 557056.0f;
+  q = fmaf(q, y, 143.0f / 10240.0f);
+  q = fmaf(q, y, 231.0f / 13312.0f);
+  q = fmaf(q, y, 63.0f / 2816.0f);
+  double p = high64(q);
   p = fma(p, z, 35.0 / 1152.0);
   p = fma(p, z, 5.0 / 112.0);
   p = fma(p, z, 3.0 / 40.0);
@@ -70,23 +91,23 @@ __device__ __forceinline__ double asin_series64(double t) {
   return fma(t * z, p, t);
 }
 
-// (1/2) log1p(s) = atanh(s / (2 + s)) for |s| < 1/16, truncated below 2^-60
+// (1/2) log1p(s) = atanh(t), t = s / (2 + s), for |s| < 1/16, truncated below
+// 2^-60; FP32 from t^8 on (2^-43 of t)
 __device__ __forceinline__ double half_log1p64(double s) {
   if (!((hi_word(s) & 0x7fffffff) < 0x3fb00000)) return 0.5 * log1p(s);
   const double t = s * recip64(2.0 + s), z = t * t;
-  double p = 1.0 / 11.0;
-  p = fma(p, z, 1.0 / 9.0);
+  const float y = low32(z);
+  double p = high64(fmaf(1.0f / 11.0f, y, 1.0f / 9.0f));
   p = fma(p, z, 1.0 / 7.0);
   p = fma(p, z, 1.0 / 5.0);
   p = fma(p, z, 1.0 / 3.0);
   return fma(t * z, p, t);
 }
 
-// exp(x) for |x| <= 1/32, truncated below 2^-60
+// exp(x) for |x| <= 1/32, truncated below 2^-60; FP32 from x^6 on (2^-39)
 __device__ __forceinline__ double exp_series64(double x) {
-  double p = 1.0 / 40320.0;
-  p = fma(p, x, 1.0 / 5040.0);
-  p = fma(p, x, 1.0 / 720.0);
+  const float y = low32(x);
+  double p = high64(fmaf(fmaf(1.0f / 40320.0f, y, 1.0f / 5040.0f), y, 1.0f / 720.0f));
   p = fma(p, x, 1.0 / 120.0);
   p = fma(p, x, 1.0 / 24.0);
   p = fma(p, x, 1.0 / 6.0);
@@ -94,16 +115,16 @@ __device__ __forceinline__ double exp_series64(double x) {
   return fma(fma(p, x, 1.0), x, 1.0);
 }
 
-// sin and cos of (n, b) = node angle + b, |b| <= pi / 64
+// sin and cos of (n, b) = node angle + b, |b| <= pi / 64; FP32 for the last two
+// terms of each series (2^-38 of sin b; 2^-35)
 __device__ __forceinline__ void turn64(double2 n, double b, double &st, double &ct) {
   const double z = b * b;
-  double p = 1.0 / 362880.0, q = 1.0 / 40320.0;
-  p = fma(p, z, -1.0 / 5040.0);
-  p = fma(p, z, 1.0 / 120.0);
+  const float y = low32(z);
+  double p = high64(fmaf(-1.0f / 362880.0f, y, 1.0f / 5040.0f)), q = high64(fmaf(-1.0f / 40320.0f, y, 1.0f / 720.0f));
+  p = fma(-p, z, 1.0 / 120.0);
   p = fma(p, z, -1.0 / 6.0);
   const double sb = fma(b * z, p, b);
-  q = fma(q, z, -1.0 / 720.0);
-  q = fma(q, z, 1.0 / 24.0);
+  q = fma(-q, z, 1.0 / 24.0);
   q = fma(q, z, -0.5);
   const double cb1 = q * z;  // cos b - 1
   st = fma(n.y, sb, fma(n.x, cb1, n.x));
@@ -342,9 +363,10 @@ __global__ void __launch_bounds__(256) k_particles64(const __grid_constant__ Arg
     // where it crosses grid lines
     const double d1 = nx1 - x1, d2 = nx2 - x2;
     double mx = fma(0.5, d1, dx), my = fma(0.5, d2, dy);  // the path's midpoint in the old cell's frame
-    if ((kx | ky) == 0) {
-      vb_seg64(D.Fr, D.Ft, o, LD, qw, dx, dy, d1, d2);
-    } else {
+    // the last segment, the only one of most paths: one code for all lanes
+    double px = dx, py = dy, q1 = d1, q2 = d2;
+    size_t om = o;
+    if (kx | ky) {
       const double ex = nx1 - fni, ey = nx2 - fnj;  // end point in the new cell's frame
       const double Xo = kx > 0 ? 1.0 : 0.0, Xn = 1.0 - Xo, Yo = ky > 0 ? 1.0 : 0.0, Yn = 1.0 - Yo;
       double sx = 2.0, sy = 2.0;  // crossing parameters, 0 to 1 (2: no crossing)
@@ -352,21 +374,23 @@ __global__ void __launch_bounds__(256) k_particles64(const __grid_constant__ Arg
       if (ky) sy = (Yo - dy) * recip64(d2);
       const bool xf = __double_as_longlong(sx) <= __double_as_longlong(sy);
       // first crossing, in the old cell's frame; the middle cell and its entry point
-      const double c1 = clamp01(xf ? fma(sx, d2, dy) : fma(sy, d1, dx)), c1x = xf ? Xo : c1, c1y = xf ? c1 : Yo;
+      const double c1 = clamp01(fma(xf ? sx : sy, xf ? d2 : d1, xf ? dy : dx)), c1x = xf ? Xo : c1, c1y = xf ? c1 : Yo;
       vb_seg64(D.Fr, D.Ft, o, LD, qw, dx, dy, c1x - dx, c1y - dy);
-      double px = xf ? Xn : c1x, py = xf ? c1y : Yn;
-      size_t om = o + (size_t)((ptrdiff_t)(xf ? kx : 0) * LD + (xf ? 0 : ky));
-      const size_t oe = o + (size_t)((ptrdiff_t)kx * LD + ky);
+      px = xf ? Xn : c1x;
+      py = xf ? c1y : Yn;
+      om = o + (size_t)((ptrdiff_t)(xf ? kx : 0) * LD + (xf ? 0 : ky));
       if (kx && ky) {  // second crossing, in the middle cell's frame
-        const double c2 = clamp01(xf ? fma(sy - 1.0, d1, ex) : fma(sx - 1.0, d2, ey)), c2x = xf ? c2 : Xo,
+        const double c2 = clamp01(fma((xf ? sy : sx) - 1.0, xf ? d1 : d2, xf ? ex : ey)), c2x = xf ? c2 : Xo,
                      c2y = xf ? Yo : c2;
         vb_seg64(D.Fr, D.Ft, om, LD, qw, px, py, c2x - px, c2y - py);
         px = xf ? c2x : Xn;
         py = xf ? Yn : c2y;
-        om = oe;
+        om = o + (size_t)((ptrdiff_t)kx * LD + ky);
       }
-      vb_seg64(D.Fr, D.Ft, om, LD, qw, px, py, ex - px, ey - py);
+      q1 = ex - px;
+      q2 = ey - py;
     }
+    vb_seg64(D.Fr, D.Ft, om, LD, qw, px, py, q1, q2);
     // azimuthal flux: charge crossing the meridional half-plane, area weights
     // at the midpoint of the grid-coordinate path (reading of the paper)
     size_t oa = o;
