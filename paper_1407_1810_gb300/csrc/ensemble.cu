@@ -259,9 +259,14 @@ static int ensemble_batched(pic_ctx *const *ctxs, int n, int nsteps, int64_t *ke
       for (int st = 0; st < block; ++st) {
         const EnsFieldArg *dfa = reinterpret_cast<const EnsFieldArg *>(d_tab + (size_t)st * step_sz);
         const StepTiles &T = tiles[st];
+        bool first = true;
         for (int kind = 0; kind < ENS_TILE_KINDS; ++kind)
-          if (!T.blocks[kind].empty())
-            nodes += ens_tiles32(kind, T.arg[kind].data(), T.blocks[kind].data(), (int)T.blocks[kind].size(), origin);
+          if (!T.blocks[kind].empty()) {
+            const int k = ens_tiles32(kind, T.arg[kind].data(), T.blocks[kind].data(), (int)T.blocks[kind].size(), origin,
+                                      first);
+            nodes += k;
+            first = first && k == 0;
+          }
         if (maps.blocks(L_FLUX) > 0) ens_flux(dfa, L(L_FLUX), maps.blocks(L_FLUX), origin), ++nodes;
         for (int p = 0; p < max_filt; ++p)
           if (maps.blocks(L_FILT + p) > 0) ens_filter(dfa, L(L_FILT + p), maps.blocks(L_FILT + p), p, origin), ++nodes;

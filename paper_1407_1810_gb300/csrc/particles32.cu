@@ -663,7 +663,15 @@ void ens_tile_arg(pic_ctx *c, double t, void *out) {
   memcpy(out, &a, sizeof a);
 }
 
-int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaStream_t s) {
+// The tile launches of one step of an ensemble (members in batches of
+// ENS_TILE_SLOTS, one kind after the other) touch different members: each but
+// the first starts as soon as the one before it has its last blocks on the
+// chip, and ends after it, so what follows waits for all of them.  Only the
+// first waits for the step before it, by plain stream order; the later ones
+// start after the first's blocks, hence after that wait too.
+// 64 members, two launches a step: 50.2 -> 49.3 ms for 40 steps (the first's
+// last, partly filled round of the chip is shared with the second).
+int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaStream_t s, bool first_of_step) {
   const EnsTileArg *T = static_cast<const EnsTileArg *>(args);
   const bool pack = kind >= 9;
   const int spec = kind % 9 / 3, shape = kind % 3;
@@ -678,7 +686,7 @@ int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaSt
       B.off[k + 1] = B.off[k] + (int)blocks[first + k];
     }
     const unsigned g = (unsigned)B.off[m];
-    (pack ? launch_ens_two : launch_ens_one)(spec, shape, g, s, B);
+    (pack ? launch_ens_two : launch_ens_one)(spec, shape, g, s, !first_of_step || launches > 0, B);
     ++launches;
   }
   return launches;

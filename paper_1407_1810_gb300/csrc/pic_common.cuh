@@ -26,6 +26,7 @@ namespace pic {
 // cost it more than they gain (64 x 64 FP64 step 101 us without overlap, 123
 // with the early start, 91 so; 72 x 56 FP32 40.6, 34.7, 30.5; 192 x 160 56.2,
 // 56.7, 46; 250 x 231 84, -, 75).
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void follow() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Launch k on s; with overlap, as a dependent of the kernel launched before it

@@ -246,7 +246,7 @@ void ens_tile_arg(pic_ctx *c, double t, void *out);  // the member's tile-kernel
 // launches the tile kernel of one kind over n members (host array of their
 // arguments, ens_tile_arg_bytes() each, and their block counts); returns the
 // number of kernels launched (members are taken in groups of up to 48)
-int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaStream_t s);
+int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaStream_t s, bool first_of_step);
 // the tile sort of m FP32 contexts at once on stream st (each launch serves
 // every member; one read-back, one synchronisation); the staging buffers
 // persist in sc between calls.  *kernels: the kernels launched.

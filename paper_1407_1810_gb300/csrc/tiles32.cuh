@@ -189,8 +189,8 @@ void launch_one(int spec, int shape, unsigned blocks, cudaStream_t s, bool overl
                 const TileMaps &M);
 void launch_two(int spec, int shape, unsigned blocks, cudaStream_t s, bool overlap, const Args32 &A, const Parts32 &P,
                 const TileMaps &M);
-void launch_ens_one(int spec, int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &B);
-void launch_ens_two(int spec, int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &B);
+void launch_ens_one(int spec, int shape, unsigned blocks, cudaStream_t s, bool beside, const EnsTileBatch &B);
+void launch_ens_two(int spec, int shape, unsigned blocks, cudaStream_t s, bool beside, const EnsTileBatch &B);
 
 }  // namespace t32
 }  // namespace pic

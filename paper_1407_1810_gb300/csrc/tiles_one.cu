@@ -556,9 +556,11 @@ __global__ void __launch_bounds__(NT, 4) k_tiles32(Args32 A, Parts32 P, const __
   tiles32_block<TI, TJ, SPEC, false>(A, P, maps.m, blockIdx.x);
 }
 
-// the tile kernel over several members of an ensemble in one grid
+// the tile kernel over several members of an ensemble in one grid; see
+// ens_tiles32 for what its launches do to each other
 template <int TI, int TJ, int SPEC>
 __global__ void __launch_bounds__(NT, 4) k_ens_tiles32(const __grid_constant__ EnsTileBatch B) {
+  next_may_start();
   int lo = 0, hi = B.n - 1;  // the member owning this block
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -567,6 +569,7 @@ __global__ void __launch_bounds__(NT, 4) k_ens_tiles32(const __grid_constant__ E
   }
   const EnsTileArg &T = B.a[lo];
   tiles32_block<TI, TJ, SPEC, true>(T.A, T.P, T.maps, blockIdx.x - (unsigned)B.off[lo]);
+  follow();
 }
 
 template <int SPEC>
@@ -577,10 +580,10 @@ void launch(int shape, unsigned blocks, cudaStream_t s, bool overlap, const Args
 }
 
 template <int SPEC>
-void launch_ens(int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &B) {
-  if (shape == 1) k_ens_tiles32<8, 32, SPEC><<<blocks, NT, 0, s>>>(B);
-  else if (shape == 2) k_ens_tiles32<32, 8, SPEC><<<blocks, NT, 0, s>>>(B);
-  else k_ens_tiles32<16, 16, SPEC><<<blocks, NT, 0, s>>>(B);
+void launch_ens(int shape, unsigned blocks, cudaStream_t s, bool beside, const EnsTileBatch &B) {
+  if (shape == 1) launch_on(s, beside, k_ens_tiles32<8, 32, SPEC>, blocks, NT, B);
+  else if (shape == 2) launch_on(s, beside, k_ens_tiles32<32, 8, SPEC>, blocks, NT, B);
+  else launch_on(s, beside, k_ens_tiles32<16, 16, SPEC>, blocks, NT, B);
 }
 
 }  // namespace
@@ -592,10 +595,11 @@ void launch_one(int spec, int shape, unsigned blocks, cudaStream_t s, bool overl
   else launch<SPEC_GENERIC>(shape, blocks, s, overlap, A, P, M);
 }
 
-void launch_ens_one(int spec, int shape, unsigned blocks, cudaStream_t s, const EnsTileBatch &B) {
-  if (spec == SPEC_MONOPOLE) launch_ens<SPEC_MONOPOLE>(shape, blocks, s, B);
-  else if (spec == SPEC_ROTATOR) launch_ens<SPEC_ROTATOR>(shape, blocks, s, B);
-  else launch_ens<SPEC_GENERIC>(shape, blocks, s, B);
+void launch_ens_one(int spec, int shape, unsigned blocks, cudaStream_t s, bool beside,
+                    const EnsTileBatch &B) {
+  if (spec == SPEC_MONOPOLE) launch_ens<SPEC_MONOPOLE>(shape, blocks, s, beside, B);
+  else if (spec == SPEC_ROTATOR) launch_ens<SPEC_ROTATOR>(shape, blocks, s, beside, B);
+  else launch_ens<SPEC_GENERIC>(shape, blocks, s, beside, B);
 }
 
 }  // namespace t32
