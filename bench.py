@@ -163,7 +163,7 @@ def recorded_traffic():
     """DRAM bytes per particle of the tile kernel from the committed ncu
     summary, if the kernel source has not changed since it was taken."""
     p = os.path.join(ROOT, "profiles", "k_tiles32_traffic.json")
-    src = os.path.join(ROOT, "paper_1407_1810_gb300", "csrc", "particles32.cu")
+    src = os.path.join(ROOT, "paper_1407_1810_gb300", "csrc", "tiles_two.cu")
     if not os.path.exists(p):
         return None
     d = json.load(open(p))

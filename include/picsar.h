@@ -245,8 +245,9 @@ int pic_set_clock(pic_ctx *c, int64_t step, int64_t next_id);
 
 /* Per-kernel timing of later steps with CUDA events on the context's stream:
  * enable = 1 starts accumulating; pic_get_profile writes the mean milliseconds
- * per launch of [particle kernel, deposit reduction, filter, field update,
- * injection, sort] into ms6 and the number of timed steps into *steps. */
+ * per launch of [particle kernel, 0, 0, grid update, injection, sort] into ms6
+ * and the number of timed steps into *steps.  The grid update holds the filter
+ * and both Yee kernels (slots 1 and 2 timed kernels that are part of it). */
 int pic_profile(pic_ctx *c, int32_t enable);
 int pic_get_profile(pic_ctx *c, double *ms6, int64_t *steps);
 
@@ -289,9 +290,9 @@ int pic_get_launches(pic_ctx *c, int64_t *n);
  *
  * All FP32 members: each phase of a step is ONE kernel launch over the blocks
  * of every member that takes part in it -- the tile kernel once per tile
- * shape and specialisation present, then the flux conversion, each filter
- * pass, the three Yee sub-steps, the lossy layer, the axis ghosts and FP32
- * copies, and the injection phases -- with the members' arguments for each
+ * shape, specialisation and form present, then the E update (with up to four
+ * filter passes; more run one launch each, after a flux conversion), the B
+ * update, and the injection phases -- with the members' arguments for each
  * step in a device table; the steps up to the next sort of any member are
  * captured into one CUDA graph, launched once.  Each member's tile sort runs
  * between graphs when its own sort interval comes due, so every member takes

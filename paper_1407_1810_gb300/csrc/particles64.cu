@@ -191,7 +191,8 @@ __device__ __forceinline__ void add_vacuum64(const Grid &G, double r0W, double i
   }
 }
 
-// Vay (2008) and Boris (1970) pushes, Sec. 2 (as push_vay and push_boris)
+// Vay (2008) and Boris (1970) pushes, Sec. 2, in a right-handed orthonormal
+// basis; qmdt = (q / m) dt, u = gamma v updated in place
 __device__ __forceinline__ void vay64(double qmdt, const double E[3], const double B[3], double u[3]) {
   const double h = 0.5 * qmdt;
   const double ig0 = rsqrt64(fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], 1.0))));

@@ -173,19 +173,15 @@ __device__ inline double map_r(const Grid &G, double x1) {
 __device__ inline double map_r_inv(const Grid &G, double r) {
   return G.r_map == 1 ? log(r / G.r_min) / G.dxi : (r - G.r_min) / G.dxi;
 }
-__device__ inline double map_th(const Grid &G, double x2) {
-  return G.th_map == 1 ? acos(1.0 - 2.0 * x2 / G.nth) : PI_D * x2 / G.nth;
-}
 __device__ inline double map_th_inv(const Grid &G, double th) {
   return G.th_map == 1 ? 0.5 * G.nth * (1.0 - cos(th)) : th * G.nth / PI_D;
 }
 
-// reciprocal and reciprocal square root: hardware approximations (within 2
-// ulp) in FP32, exact division in FP64
+// reciprocal (exact division in FP64) and reciprocal square root: hardware
+// approximations (within 2 ulp) in FP32
 __device__ inline float rcp_(float x) { return __fdividef(1.0f, x); }
 __device__ inline double rcp_(double x) { return 1.0 / x; }
 __device__ inline float rsqrt_(float x) { return rsqrtf(x); }
-__device__ inline double rsqrt_(double x) { return 1.0 / sqrt(x); }
 
 // ---- analytic "initial" fields: Sec. 5.2 (monopole, rotator inside/outside),
 //      Sec. 4.3 (dipole + corotation), uniform B_z.  Spherical components.
@@ -249,51 +245,6 @@ __device__ inline void vacuum_field(const Vac<T> &V, T r, T st, T ct, bool insid
     default:
       break;
   }
-}
-
-// ---- pushers, Sec. 2 (Boris 1970; Vay 2008).  Any right-handed orthonormal
-//      basis; qmdt = (q/m) dt.  u = gamma v updated in place. -------------------
-template <typename T>
-__device__ inline void push_boris(T qmdt, const T E[3], const T B[3], T u[3]) {
-  const T h = T(0.5) * qmdt;
-  T um0 = u[0] + h * E[0], um1 = u[1] + h * E[1], um2 = u[2] + h * E[2];
-  T ig = rsqrt_(T(1) + um0 * um0 + um1 * um1 + um2 * um2);
-  T t0 = h * B[0] * ig, t1 = h * B[1] * ig, t2 = h * B[2] * ig;
-  T f = T(2) * rcp_(T(1) + t0 * t0 + t1 * t1 + t2 * t2);
-  T up0 = um0 + (um1 * t2 - um2 * t1), up1 = um1 + (um2 * t0 - um0 * t2), up2 = um2 + (um0 * t1 - um1 * t0);
-  T s0 = f * t0, s1 = f * t1, s2 = f * t2;
-  u[0] = um0 + (up1 * s2 - up2 * s1) + h * E[0];
-  u[1] = um1 + (up2 * s0 - up0 * s2) + h * E[1];
-  u[2] = um2 + (up0 * s1 - up1 * s0) + h * E[2];
-}
-
-template <typename T>
-__device__ inline void push_vay(T qmdt, const T E[3], const T B[3], T u[3]) {
-  const T h = T(0.5) * qmdt;
-  T ig0 = rsqrt_(T(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-  T tau0 = h * B[0], tau1 = h * B[1], tau2 = h * B[2];
-  T v0 = u[0] * ig0, v1 = u[1] * ig0, v2 = u[2] * ig0;
-  // u' = u + (q dt/m) E + v x tau
-  T a0 = u[0] + qmdt * E[0] + (v1 * tau2 - v2 * tau1);
-  T a1 = u[1] + qmdt * E[1] + (v2 * tau0 - v0 * tau2);
-  T a2 = u[2] + qmdt * E[2] + (v0 * tau1 - v1 * tau0);
-  T tau2s = tau0 * tau0 + tau1 * tau1 + tau2 * tau2;
-  T ustar = a0 * tau0 + a1 * tau1 + a2 * tau2;
-  T sigma = T(1) + a0 * a0 + a1 * a1 + a2 * a2 - tau2s;
-  T g2 = T(0.5) * (sigma + sqrt(sigma * sigma + T(4) * (tau2s + ustar * ustar)));
-  T ig = rsqrt_(g2);
-  T t0 = tau0 * ig, t1 = tau1 * ig, t2 = tau2 * ig;
-  T s = rcp_(T(1) + t0 * t0 + t1 * t1 + t2 * t2);
-  T at = a0 * t0 + a1 * t1 + a2 * t2;
-  u[0] = s * (a0 + at * t0 + (a1 * t2 - a2 * t1));
-  u[1] = s * (a1 + at * t1 + (a2 * t0 - a0 * t2));
-  u[2] = s * (a2 + at * t2 + (a0 * t1 - a1 * t0));
-}
-
-template <typename T>
-__device__ inline void push(int pusher, T qmdt, const T E[3], const T B[3], T u[3]) {
-  if (pusher == 1) push_boris(qmdt, E, B, u);
-  else push_vay(qmdt, E, B, u);
 }
 
 // ---- ties of the azimuth branch at the polar axis (Sec. 3.3, reading of the
