@@ -87,7 +87,6 @@ __device__ __forceinline__ void e_node(const EnsFieldArg &S, int i, int j, doubl
 // B at integer time and at the next half step of node (i, j), the axis
 // continuation of the half-integer-j components into columns -1 and nth (B_r
 // even; E_th, B_ph odd) and the FP32 gather copies of the six components.
-// SIGMA: the row at the star also forms the injection's surface charge.
 template <bool FP32>
 __device__ __forceinline__ void b_node(const EnsFieldArg &S, int i, int j) {
   const Grid &G = S.G;

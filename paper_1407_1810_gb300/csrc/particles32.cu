@@ -490,16 +490,16 @@ __global__ void k_reduce32(Parts32 P, int64_t n, double qm, double *acc, long lo
 constexpr int TRW_WARP = 32;
 
 // The form of the tile kernel a context takes.  Two particles a thread are the
-// faster form once there are tiles enough to fill the chip (1024 x 1024
-// monopole, 6.3e7 particles: 1.30 ms a step with one, 1.03 with two; rotator,
-// 1e8: 2.27 and 1.60; a whole run of 448 x 416: 11.7 and 10.6 ms); on a small
-// grid, bound by latency and by the grid phase, the two run alike (20 steps:
-// 72 x 56 rotator 0.91 and 0.93 ms, 192 x 160 dipole 1.65 and 1.64, 250 x 231
-// monopole 1.90 and 1.81; 64-member ensemble, 40 steps: 62 and 59).  They
-// round differently, and the sparse plasmas run on small grids (ensemble
-// members of a few particles a cell) amplify a rounding a hundredfold in
-// eighty steps: those keep the form and the bits they had.  The grid alone
-// decides, so that a member, a slab and a run of its own agree.
+// faster form once there are tiles enough to fill the chip (1024 x 1024, 20
+// steps: monopole of 6.3e7 particles 29.5 ms with one, 24.1 with two; rotator of
+// 1e8 49.6 and 36.9; a whole run of 448 x 416: 8.05 and 7.38); on a small grid,
+// bound by latency and by the grid phase, the two are closer (72 x 56 rotator
+// 0.65 and 0.67 ms, 192 x 160 dipole 1.35 and 1.27, 250 x 231 monopole 1.51 and
+// 1.41; 64-member ensemble, 40 steps: 49.1 and 46.8).  They round differently,
+// and the sparse plasmas run on small grids (ensemble members of a few particles
+// a cell) amplify a rounding a hundredfold in eighty steps: those keep the form
+// and the bits they had.  The grid alone decides, so that a member, a slab and a
+// run of its own agree.
 constexpr int64_t PACK_CELLS = 1 << 17;
 bool use_packed(const pic_ctx *c) { return (int64_t)c->G.nr_glob * c->G.nth > PACK_CELLS; }
 

@@ -20,7 +20,7 @@ namespace {
 // approximations; compares are made on the integer halves of a double.
 // Measured on 512 x 512, 2e7 particles: 634 FP64 instructions a particle and
 // 22.6 ms a step with exp, log, sincos, atan2, hypot and divisions in global
-// coordinates; 300 and 11.2 ms so; 10.7 ms with FP32 last terms of the series
+// coordinates; 300 and 11.2 ms so; 285 and 10.7 ms with FP32 last terms of the series
 // and one code for the last path segment of crossing and other lanes (the FP64
 // pipe at its 86 % limit throughout).
 // The local form is also the more exact one: against 50 digits, a move's
