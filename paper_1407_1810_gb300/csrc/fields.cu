@@ -274,22 +274,42 @@ constexpr int TW = BX + 2 * FUSE_FILT, TH = BY + 2 * FUSE_FILT;
 __constant__ int FILT_W[FUSE_FILT + 1][FUSE_FILT + 1] = {  // C(2N, N + k)
     {1, 0, 0, 0, 0}, {2, 1, 0, 0, 0}, {6, 4, 1, 0, 0}, {20, 15, 6, 1, 0}, {70, 56, 28, 8, 1}};
 
-// FP64 tiles take the weights from a table of doubles and the factors through
-// the exponent and sign bits: an integer-to-double conversion or a product
-// costs as much of the FP64 pipe as an addition of the convolution.
+// FP64 tiles take the weights over 4^N a direction from a table of doubles (an
+// integer-to-double conversion or a product costs as much of the FP64 pipe as
+// an addition of the convolution), so that no weighted sum is larger than what
+// it averages (only two neighbours of one sign beyond 2^1023 still overflow).
+// Where a tile holds a pole, its other nodes are halved instead of the pole's
+// doubled, so that a value of the last binade stays finite; the halving goes
+// through the exponent bits, and infinities and NaN pass as they are.  All of
+// it is exact above the subnormal numbers.
 __constant__ double FILT_WD[FUSE_FILT + 1][FUSE_FILT + 1] = {
-    {1, 0, 0, 0, 0}, {2, 1, 0, 0, 0}, {6, 4, 1, 0, 0}, {20, 15, 6, 1, 0}, {70, 56, 28, 8, 1}};
+    {1, 0, 0, 0, 0},
+    {2 / 4., 1 / 4., 0, 0, 0},
+    {6 / 16., 4 / 16., 1 / 16., 0, 0},
+    {20 / 64., 15 / 64., 6 / 64., 1 / 64., 0},
+    {70 / 256., 56 / 256., 28 / 256., 8 / 256., 1 / 256.}};
 template <class T>
 __device__ __forceinline__ T filt_weight(int N, int k) { return T(FILT_W[N][k]); }
 template <>
 __device__ __forceinline__ double filt_weight<double>(int N, int k) { return FILT_WD[N][k]; }
+// a loaded value with the factor c of its image; FP64: its sign, and half of
+// it where c stands for 1 against the 2 of a pole in the same tile
 template <class T>
-__device__ __forceinline__ T filt_scaled(int c, T v) { return T(c) * v; }
+__device__ __forceinline__ T filt_scaled(int c, bool, T v) { return T(c) * v; }
 template <>
-__device__ __forceinline__ double filt_scaled<double>(int c, double v) {
+__device__ __forceinline__ double filt_scaled<double>(int c, bool halve, double v) {
   int hi = __double2hiint(v);
-  if ((c == 2 || c == -2) && (hi & 0x7ff00000) != 0) hi += 0x00100000;  // doubled (zeros stay)
-  return __hiloint2double(c < 0 ? hi ^ 0x80000000 : hi, __double2loint(v));
+  const int lo = __double2loint(v);
+  if (halve && (c == 1 || c == -1)) {
+    const unsigned e = (unsigned)hi >> 20 & 0x7ffu;
+    if (e - 2u < 0x7fdu) {  // its half is normal
+      hi -= 0x00100000;
+    } else if (e < 2u && ((hi & 0x7fffffff) | lo)) {
+      v *= 0.5;
+      return c < 0 ? -v : v;
+    }
+  }
+  return __hiloint2double(c < 0 ? hi ^ 0x80000000 : hi, lo);
 }
 
 // Images of the rows and columns that this thread loads of a tile: array
@@ -301,6 +321,11 @@ __device__ __forceinline__ double filt_scaled<double>(int c, double v) {
 struct FiltImages {
   int row[2], row_c[2], col[2][2], col_c[2][2];
 };
+
+// whether a pole is among the columns a tile reads
+__device__ __forceinline__ bool filt_poles(const Grid &G, int j0, int N) {
+  return j0 - N <= 0 || j0 + BX - 1 + N >= G.nth;
+}
 
 __device__ __forceinline__ FiltImages filt_images(const Grid &G, int i0, int j0, int N) {
   FiltImages im;
@@ -332,10 +357,11 @@ struct FiltTile {
 };
 
 // NC components (the first of them component c0) of the tile with N passes at
-// this thread's node; every thread of the block calls it
+// this thread's node; every thread of the block calls it.  halve (FP64): the
+// tile holds a pole; the integer-j sums of its other nodes are half of theirs
 template <int N, class T, int NC, class L>
-__device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &im, const Grid &G, int c0, T out[NC],
-                                          const L &load) {
+__device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &im, const Grid &G, int c0, bool halve,
+                                          T out[NC], const L &load) {
   const int tx = threadIdx.x, ty = threadIdx.y;
   constexpr int w = BX + 2 * N, h = BY + 2 * N;
 #pragma unroll
@@ -348,7 +374,7 @@ __device__ __forceinline__ void filt_conv(FiltTile<T, NC> &t, const FiltImages &
         if (r < h && q < w) {
           const int ro = im.row[a];
           t.in[k][r][q] = ro < 0 ? T(0)
-                                 : filt_scaled<T>(im.row_c[a] * im.col_c[half][b],
+                                 : filt_scaled<T>(im.row_c[a] * im.col_c[half][b], halve && !half,
                                                   load(c0 + k, (size_t)ro * G.LD + im.col[half][b]));
         }
       }
@@ -394,7 +420,7 @@ __device__ __forceinline__ void filtered_flux(const EnsFieldArg &S, FiltSmem &sm
     const long long lim = 1ll << (60 - 4 * N);
     bool big = false;
     long long v[3];
-    filt_conv<N>(sm.q, im, G, 0, v, [&](int k, size_t x) {
+    filt_conv<N>(sm.q, im, G, 0, false, v, [&](int k, size_t x) {
       const long long y = S.acc[k][x];
       big |= y >= lim || y <= -lim;
       return y;
@@ -404,17 +430,17 @@ __device__ __forceinline__ void filtered_flux(const EnsFieldArg &S, FiltSmem &sm
     if (__syncthreads_or(big)) {
       for (int k = 0; k < 3; ++k) {
         __int128 z[1];
-        filt_conv<N>(sm.w, im, G, k, z, [&](int c, size_t x) { return (__int128)S.acc[c][x]; });
+        filt_conv<N>(sm.w, im, G, k, false, z, [&](int c, size_t x) { return (__int128)S.acc[c][x]; });
         F[k] = fixed_to_f64(k != 1 && pole ? z[0] / 2 : z[0], s - 4 * N);
         __syncthreads();
       }
     }
   } else {
-    const double sc = __longlong_as_double((long long)(1023 - 4 * N) << 52);  // 16^-N
     double v[3];
-    filt_conv<N>(sm.d, im, G, 0, v, [&](int k, size_t x) { return S.Fin[k][x]; });
+    const bool poles = filt_poles(G, j0, N);
+    filt_conv<N>(sm.d, im, G, 0, poles, v, [&](int k, size_t x) { return S.Fin[k][x]; });
 #pragma unroll
-    for (int k = 0; k < 3; ++k) F[k] = v[k] * (k != 1 && pole ? 0.5 * sc : sc);
+    for (int k = 0; k < 3; ++k) F[k] = k != 1 && poles && !pole ? v[k] + v[k] : v[k];
   }
 }
 
@@ -478,22 +504,22 @@ __device__ __forceinline__ void b_block(const EnsFieldArg &S, unsigned b, bool s
 
 // the passes of an integer-j FP64 array (the node charge) in one
 template <int N>
-__device__ __forceinline__ double filtered_charge(FiltTile<double, 1> &t, const Grid &G, int i0, int j0,
+__device__ __forceinline__ double filtered_charge(FiltTile<double, 1> &t, const Grid &G, int i0, int j0, bool pole,
                                                   const double *__restrict__ a) {
   double v[1];
-  filt_conv<N>(t, filt_images(G, i0, j0, N), G, 0, v, [&](int, size_t x) { return a[x]; });
-  return v[0];
+  const bool poles = filt_poles(G, j0, N);
+  filt_conv<N>(t, filt_images(G, i0, j0, N), G, 0, poles, v, [&](int, size_t x) { return a[x]; });
+  return poles && !pole ? v[0] + v[0] : v[0];
 }
 __global__ void __launch_bounds__(BX *BY) k_filter_tile(Grid G, const double *__restrict__ a, double *__restrict__ out,
                                                        int N) {
   __shared__ FiltTile<double, 1> t;
   const int i0 = -G.g + (int)blockIdx.y * BY, j0 = (int)blockIdx.x * BX;
-  const double v = N == 1 ? filtered_charge<1>(t, G, i0, j0, a) : N == 2 ? filtered_charge<2>(t, G, i0, j0, a)
-                 : N == 3 ? filtered_charge<3>(t, G, i0, j0, a) : filtered_charge<4>(t, G, i0, j0, a);
   const int i = i0 + (int)threadIdx.y, j = j0 + (int)threadIdx.x;
-  if (i > G.nr + G.g || j > G.nth) return;
-  const double sc = __longlong_as_double((long long)(1023 - 4 * N) << 52);  // 16^-N
-  out[gidx(G, i, j)] = v * (j == 0 || j == G.nth ? 0.5 * sc : sc);
+  const bool pole = j == 0 || j == G.nth;
+  const double v = N == 1 ? filtered_charge<1>(t, G, i0, j0, pole, a) : N == 2 ? filtered_charge<2>(t, G, i0, j0, pole, a)
+                 : N == 3 ? filtered_charge<3>(t, G, i0, j0, pole, a) : filtered_charge<4>(t, G, i0, j0, pole, a);
+  if (i <= G.nr + G.g && j <= G.nth) out[gidx(G, i, j)] = v;
 }
 
 template <bool FP32>
