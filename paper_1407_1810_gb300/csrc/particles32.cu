@@ -710,19 +710,25 @@ int ens_tiles32(int kind, const void *args, const int64_t *blocks, int n, cudaSt
 // Members of an ensemble share the chip: their units follow the particles of
 // all of them (64 members, 2.4e7 particles: 62 ms for 40 steps with units of
 // 4096, 64 with 2048, 71 with 1024, 78 with 512).
+// A unit is also what one CTA's 32-bit sums must hold: it never exceeds
+// UNIT_ROOM particles (which no crowding can overflow), or 1 / 1216 of a larger
+// run's.  On grids of one or a few tiles the cut goes beyond 64 pieces a tile, to
+// four rounds of the chip (20 steps of 16 x 16 cells and 1e6 particles 2.67 ms
+// with at most 64 pieces, 1.06 so; 4e6 10.0 and 3.0; 32 x 32 and 1e7 7.5 and 5.3).
 constexpr int SLOTS = 4 * 152;
 static int64_t unit_size(const pic_ctx *c) {
   const int64_t n = c->n_used;
+  const int64_t room = std::max<int64_t>(UNIT_ROOM, (n + 2 * SLOTS - 1) / (2 * SLOTS));
   if (c->ens_particles > 0) {
     const int64_t u = (c->ens_particles + 8 * SLOTS - 1) / (8 * SLOTS);
-    return std::max<int64_t>(2 * NT, (u + NT - 1) / NT * NT);
+    return std::min(room, std::max<int64_t>(2 * NT, (u + NT - 1) / NT * NT));
   }
   const Tiles &T = c->tiles;
   const int64_t tiles = (int64_t)((c->G.nr + T.TI - 1) / T.TI) * T.ntj;  // those of the grid proper
   const double avg = (double)n / (double)tiles;
   double best = 1e300;
   int64_t unit = NT;
-  for (int m = 1; m <= 64; ++m) {
+  for (int64_t m = 1; m <= 64 || m * tiles <= 4 * SLOTS; ++m) {
     const double share = avg / m;
     const double cost = std::ceil((double)m * tiles / SLOTS) * (std::ceil(share / NT) + 1.5);
     if (cost < best) {
@@ -731,7 +737,7 @@ static int64_t unit_size(const pic_ctx *c) {
     }
     if (share <= NT) break;
   }
-  return std::max(unit, (n + 4 * SLOTS - 1) / (4 * SLOTS));
+  return std::min(room, std::max(unit, (n + 4 * SLOTS - 1) / (4 * SLOTS)));
 }
 
 int64_t sort32(pic_ctx *c) {

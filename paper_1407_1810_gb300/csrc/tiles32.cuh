@@ -29,10 +29,12 @@ constexpr int NT = 256;                                  // particles per pass o
 constexpr int NTH = NT / 2;                              // its threads with two particles each
 // Shared-memory accumulation splits each term v (|v| <= 2^36 quanta) into
 // v = h 2^SPLIT + l with |h| <= 2^18, |l| <= 2^17 and sums h and l with
-// native 32-bit shared atomics: both sums stay exact below 2^31 / 2^18 = 8192
-// terms per node per tile per step (about 2000 particles per cell); sums
-// approaching that limit are reported as ERR_CAPACITY.
+// native 32-bit shared atomics.  A particle's terms on one node of a component
+// add up to at most 2^36, so the sums of a work unit of up to UNIT_ROOM
+// particles stay below 2^31 whatever they do; in a larger unit a node whose sums
+// come near that limit is reported as ERR_CAPACITY.
 constexpr int SPLIT = 18;
+constexpr int UNIT_ROOM = 8000;
 
 struct Args32 {
   int nr, nth, n_filt, PI, PJ, LD;
@@ -81,6 +83,11 @@ __device__ __forceinline__ void unit_range(const Args32 &A, long long u, int &ti
     b0 = s + n * q / m;
     b1 = s + n * (q + 1) / m;
   }
+}
+
+// whether a node's sums in a unit of n particles may have left 32 bits
+__device__ __forceinline__ bool sums_full(int hsum, int lsum, int64_t n) {
+  return (abs(hsum) >= (1 << 30) || abs(lsum) >= (1 << 30)) && n > UNIT_ROOM;
 }
 
 __device__ inline size_t pidx(const Args32 &A, int i, int j) {

@@ -536,7 +536,7 @@ __device__ __forceinline__ void tiles32_block(const Args32 &A, const Parts32 &P,
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const int hsum = shi[c * WN + e], lsum = slo[c * WN + e];
-        if (abs(hsum) >= (1 << 30) || abs(lsum) >= (1 << 30)) atomicOr(A.err, ERR_CAPACITY);  // near the limit
+        if (sums_full(hsum, lsum, b1 - b0)) atomicOr(A.err, ERR_CAPACITY);
         const long long v = ((long long)hsum << SPLIT) + (long long)lsum;
         if (v) atomicAdd(reinterpret_cast<unsigned long long *>(A.acc[c] + o), (unsigned long long)v);
       }
