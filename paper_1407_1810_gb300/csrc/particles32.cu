@@ -822,12 +822,15 @@ int ens_sort32(pic_ctx *const *cs, int m, cudaStream_t st, EnsSortScratch &sc, i
   const int nd = (int)due.size();
   if (nd == 0) return PIC_OK;
   // room for each member's work units (reallocated after the device is idle
-  // on the stream: a previous graph may still read the old list)
+  // on the stream: a previous graph may still read the old list).  A member's
+  // unit size goes with its list: until every call has succeeded it keeps both.
   bool synced = false;
-  for (pic_ctx *c : due) {
+  std::vector<int64_t> unit(nd);
+  for (int k = 0; k < nd; ++k) {
+    pic_ctx *c = due[k];
     Tiles &T = c->tiles;
-    T.unit = unit_size(c);
-    const int64_t ucap = T.ntiles + c->n_used / T.unit + 1;
+    unit[k] = unit_size(c);
+    const int64_t ucap = T.ntiles + c->n_used / unit[k] + 1;
     if (ucap <= T.units_cap) continue;
     if (!synced) { PIC_CUDA(cudaStreamSynchronize(st)); synced = true; }
     cudaFree(T.units);
@@ -852,7 +855,6 @@ int ens_sort32(pic_ctx *const *cs, int m, cudaStream_t st, EnsSortScratch &sc, i
     EnsSortArg &E = tab[k];
     E.A = make_args(c, 0.0);
     E.A.mix = c->mix_sort ? 1 : 0;
-    c->mix_sort = false;
     E.S = c->p32;
     E.D = c->q32;
     E.n = c->n_used;
@@ -867,7 +869,7 @@ int ens_sort32(pic_ctx *const *cs, int m, cudaStream_t st, EnsSortScratch &sc, i
     E.ucount = T.ucount;
     E.usum = T.usum;
     E.units = T.units;
-    E.unit = T.unit;
+    E.unit = unit[k];
     E.err = c->d_err;
     add(M_ZERO, k, (T.nbins + 1 + 255) / 256);
     add(M_PART, k, (E.n + 255) / 256);
@@ -923,7 +925,9 @@ int ens_sort32(pic_ctx *const *cs, int m, cudaStream_t st, EnsSortScratch &sc, i
     std::swap(c->p32, c->q32);
     c->n_used = out[3 * k];
     T.sorted_end = out[3 * k];
+    T.unit = unit[k];
     T.nunits = out[3 * k + 1];
+    c->mix_sort = false;
     c->host_err |= (int)out[3 * k + 2];
     c->steps_since_sort = 0;
     c->launches += 10;  // the kernels of its own sort (sort32)
