@@ -9,6 +9,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>  // CUdeviceptr
+
 #include "pic_internal.h"
 
 using namespace pic;
@@ -355,26 +357,55 @@ Planes field_planes(const pic_ctx *c) {
   return S;
 }
 
-// Whether a kernel can write n doubles at `out` itself: memory of the GPU
-// (or managed), on an 8-byte boundary.  Anything else takes a staging copy.
-bool writable_here(const pic_ctx *c, const void *out, int mem) {
-  if (mem != PIC_MEM_DEVICE || ((uintptr_t)out & 7) != 0) return false;
+// Bytes from p to the end of the device allocation that holds it; 0: not known
+size_t bytes_ahead(const void *p) {
+  using Range = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+  static const Range range = [] {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Range>(fn) : nullptr;
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (!range || range(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return 0;
+  return (size_t)(base + size - (CUdeviceptr)p);
+}
+
+// How n doubles reach `out`: a kernel writes them where it is memory of the GPU
+// (or managed), on an 8-byte boundary and in one allocation; anything else
+// takes a staging copy.  REFUSED: the memory at `out` ends before them.
+enum Route { DIRECT, STAGED, REFUSED };
+Route route_to(const pic_ctx *c, const double *out, size_t n, int mem) {
+  if (mem != PIC_MEM_DEVICE || ((uintptr_t)out & 7) != 0) return STAGED;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, out) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return STAGED;
   }
-  return (a.type == cudaMemoryTypeDevice && a.device == c->device) || a.type == cudaMemoryTypeManaged;
+  if (!((a.type == cudaMemoryTypeDevice && a.device == c->device) || a.type == cudaMemoryTypeManaged)) return STAGED;
+  const size_t bytes = n * sizeof(double);
+  size_t at = bytes_ahead(out);
+  if (at >= bytes) return DIRECT;
+  if (at == 0) return STAGED;
+  while (at < bytes) {  // a buffer mapped from several allocations in a row, or one that is too short
+    const size_t more = bytes_ahead((const char *)out + at);
+    if (more == 0) return REFUSED;
+    at += more;
+  }
+  return STAGED;
 }
 
 // Runs `fill(double *dst)` (kernels that write n doubles) into the caller's
-// buffer: directly where a kernel can write there, otherwise through the
+// buffer: directly where route_to allows it, otherwise through the
 // context's staging area or, for more than it holds, an allocation; and waits
 // for it.  (A 250 x 231 grid's fields to the device: 246 us with an allocation,
 // six launches, a copy and a free, 44 us so.)
 template <class Fill>
 int deliver(pic_ctx *c, double *out, size_t n, int mem, const Fill &fill) {
-  if (writable_here(c, out, mem)) {
+  const Route route = route_to(c, out, n, mem);
+  if (route == REFUSED) return pic_fail(PIC_ECUDA, "output buffer: invalid argument (its allocation ends before the values)");
+  if (route == DIRECT) {
     fill(out);
     PIC_CUDA(cudaGetLastError());
     PIC_CUDA(cudaStreamSynchronize(c->stream));
