@@ -251,7 +251,7 @@ int alloc_parts(pic_ctx *c, int64_t cap) {
       B.add(&p->id, n);
     }
   }
-  // scratch: block counts of the FP64 path's stable compaction
+  // scratch: block counts of the FP64 path's stable compaction; the FP32 path's list of small charges
   c->scratch_bytes = ((size_t)cap / 256 + 2) * sizeof(long long);
   B.add((char **)&c->scratch, c->scratch_bytes);
   const int e = B.allocate(&c->parts_block, false);

@@ -316,21 +316,32 @@ __global__ void k_ens_sort_out(const EnsSortArg *__restrict__ tab, int m) {
 }
 
 // ---- node charge (diagnostics) ----------------------------------------------
-// Positive and negative charge at every node, exact: a particle's |qw| in
-// units of 2^(e - QFIX) (e: the context's charge exponent) is an integer, its
-// offsets are 64-bit fractions, and the four area weights' shares are 64-bit
-// products rounded down that add up to the whole charge.  Q is their
-// difference and sum |qw| their sum, rounded once to FP64.  A block takes a
-// work unit of the tile kernel (one tile's particles, which are mixed across
-// its cells) and sums three 18-bit limbs a node in shared memory with native
-// 32-bit atomics, flushed before they can overflow; particles outside the
-// window add to global memory.  With one FP64 global atomic per node, sign and
-// particle this took 4.4 ms for the 5e7 particles of a 1024^2 rotator, bound
-// by the atomics and the FP64 pipe; 0.44 ms so.
-constexpr int QFIX = 54, QLIMB = 18, QSPLIT = 27;  // fraction bits; limb; low part of a global sum
-constexpr int QFLUSH = (1 << 13) / NT;               // passes of NT particles: 2^13 terms of at most 2^18
-struct ChargePlanes {  // sums of the high and the low QSPLIT bits, of positive and negative charge
-  unsigned long long *hi[2], *lo[2];
+// Positive and negative charge at every node.  A particle's |qw| in units of
+// 2^(e - QFIX) (e: the context's charge exponent) is an integer, its offsets are
+// 64-bit fractions, and the four area weights' shares are 64-bit products rounded
+// down that add up to the whole charge: sums of integers, in any order the same.
+// A share is off by up to 3 units, 3 2^-54 of the particle's charge while that is
+// at least 2^(e - QRANGE).  Smaller charges (other species, pairs injected where
+// the surface charge is small, an exponent that flux_quantum raised) take FP64
+// products and FP64 atomics, in a kernel of their own that leaves at once where
+// there are none.  Q is the difference of the signs' sums and sum |qw| their sum,
+// rounded once to FP64; the small charges are added to that.
+//
+// A block takes a work unit of the tile kernel (one tile's particles, which are
+// mixed across its cells) and sums three 20-bit limbs a node in shared memory with
+// native 32-bit atomics, flushed before they can overflow; particles outside the
+// window add to global memory.  5e7 particles of a 1024^2 rotator: 4.6 ms with
+// FP64 global atomics for all, bound by the atomics and the FP64 pipe; 0.54 ms so,
+// and 0.66 ms with charges that vary as |cos theta|, 3 % of them small.  (18-bit
+// limbs, half the flushes and no small charges told apart: 0.52.  19-bit, QRANGE 3:
+// 0.52, and 0.89 with 12 % small; 21-bit, QRANGE 8: 0.57 and 0.66.  The small
+// charges' atomics in the tile kernel: 0.04 more for all.)
+constexpr int QFIX = 59, QLIMB = 20, QSPLIT = 30;  // fraction bits; limb; low part of a global sum
+constexpr int QRANGE = 5;
+constexpr int QFLUSH = (1 << 12) / NT;               // passes of NT particles: 2^12 terms of less than 2^20
+struct ChargePlanes {
+  unsigned long long *hi[2], *lo[2];  // sums of the high and the low QSPLIT bits, of positive and negative charge
+  long long *list, cap;               // the slots of the first cap charges below 2^(e - QRANGE) (CNT_SMALL counts all)
 };
 
 // w in [0, 1) as a fraction of 2^64 (exact from 2^-40 on)
@@ -340,12 +351,21 @@ __device__ __forceinline__ unsigned long long frac64(float w) {
   return ex >= 86 ? m << (ex - 86) : (ex + 64 > 86 ? m >> (86 - ex) : 0ull);
 }
 
-// the charge of a particle in units of 2^(e - QFIX)
+// whether a charge lies in [2^(e - QRANGE), 2^e], and it in units of 2^(e - QFIX) if so
+__device__ __forceinline__ bool charge_fits(float q, int e) {
+  return (unsigned)((int)(__float_as_uint(q) >> 23 & 0xffu) - 127 - (e - QRANGE)) <= (unsigned)QRANGE;
+}
 __device__ __forceinline__ unsigned long long charge_units(float q, int e) {
   const unsigned b = __float_as_uint(q) & 0x7fffffffu;
-  const int sh = (int)(b >> 23) - 150 + QFIX - e;  // q = m 2^(exponent - 150)
-  const unsigned long long m = (b & 0x7fffffu) | 0x800000u;  // charges are normal numbers
-  return sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ull);
+  return (unsigned long long)((b & 0x7fffffu) | 0x800000u) << ((int)(b >> 23) - 150 + QFIX - e);  // q = m 2^(exponent - 150)
+}
+
+// particle k into the list of small charges (a list that has run over needs no
+// more of them)
+__device__ __forceinline__ void charge_list(const Args32 &A, const ChargePlanes &C, int64_t k) {
+  if (*(volatile long long *)(A.cnt + CNT_SMALL) > C.cap) return;
+  const long long at = (long long)atomicAdd((unsigned long long *)A.cnt + CNT_SMALL, 1ull);
+  if (at < C.cap) C.list[at] = k;
 }
 
 struct ChargeShare {
@@ -390,7 +410,9 @@ __global__ void __launch_bounds__(NT) k_charge_tiles(Args32 A, Parts32 P, Charge
       float dy = P.dy[k];
       if (dy >= 1.f) { dy = 0.f; ++cj; }  // on the south axis
       const int sg = q < 0.f;
-      const ChargeShare s = charge_share(charge_units(q, e), dx, dy);
+      const bool fits = charge_fits(q, e);
+      if (!fits) charge_list(A, C, k);
+      const ChargeShare s = charge_share(fits ? charge_units(q, e) : 0ull, dx, dy);
       if (binned && ci >= i0 - H && ci < i0 + TI + H && cj >= j0 - H && cj < j0 + TJ + H + 1) {
         const int o = (ci - wi0) * WJ + (cj - wj0);
 #pragma unroll
@@ -417,10 +439,11 @@ __global__ void __launch_bounds__(NT) k_charge_tiles(Args32 A, Parts32 P, Charge
       for (int w = threadIdx.x; w < 2 * WN; w += NT) {
         const int sgn = w >= WN, n = sgn ? w - WN : w;
         const unsigned long long l0 = lim[sgn][0][n], l1 = lim[sgn][1][n], l2 = lim[sgn][2][n];
-        if (l0 | l1 | l2) {  // l2 2^36 + l1 2^18 + l0 at QSPLIT = 27 bits
+        if (l0 | l1 | l2) {  // l2 2^40 + l1 2^20 + l0 at QSPLIT = 30 bits
           const size_t o = pidx(A, wi0 + n / WJ, wj0 + n % WJ);
-          atomicAdd(C.hi[sgn] + o, (l2 << 9) + (l1 >> 9));
-          atomicAdd(C.lo[sgn] + o, ((l1 & 511ull) << QLIMB) + l0);
+          constexpr int R = QSPLIT - QLIMB;
+          atomicAdd(C.hi[sgn] + o, (l2 << (QLIMB - R)) + (l1 >> R));
+          atomicAdd(C.lo[sgn] + o, ((l1 & ((1ull << R) - 1)) << QLIMB) + l0);
           lim[sgn][0][n] = lim[sgn][1][n] = lim[sgn][2][n] = 0;
         }
       }
@@ -442,6 +465,39 @@ __global__ void k_charge_finish(Grid G, const long long *qexp, ChargePlanes C, u
   borrowed[o] = 0;
   Q[o] = fixed_to_f64(p - n, s);
   Qa[o] = fixed_to_f64(p + n, s);
+}
+
+// the charges that k_charge_tiles left out, onto its results: those listed, or, of more than the
+// list holds, all that a pass over the charges finds
+__device__ __forceinline__ void charge_small(const Args32 &A, const Parts32 &P, double *Q, double *Qa, int64_t k) {
+  const uint32_t c = P.cell[k];
+  const size_t o = pidx(A, (int)(c >> 16) - CELL_BIAS, (int)(c & 0xffffu)), LD = A.LD;
+  const double q = P.qw[k], w1 = P.dx[k], w2 = P.dy[k], a = fabs(q);
+  const double w[4] = {(1 - w1) * (1 - w2), w1 * (1 - w2), (1 - w1) * w2, w1 * w2};
+#pragma unroll
+  for (int n = 0; n < 4; ++n) {
+    const size_t x = o + (n & 1) * LD + (n >> 1);
+    atomicAdd(Q + x, q * w[n]);
+    atomicAdd(Qa + x, a * w[n]);
+  }
+}
+
+__global__ void k_charge_small(Args32 A, Parts32 P, ChargePlanes C, double *Q, double *Qa) {
+  const int64_t n = A.cnt[CNT_SMALL], step = (int64_t)gridDim.x * blockDim.x;
+  int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (n <= C.cap) {
+    for (; k < n; k += step) charge_small(A, P, Q, Qa, C.list[k]);
+    return;
+  }
+  const int e = qexp_value(A.qexp);
+  for (; k < A.n_used; k += 8 * step) {
+    float q[8];  // the loads of eight before the first is looked at
+#pragma unroll
+    for (int r = 0; r < 8; ++r) q[r] = k + r * step < A.n_used ? P.qw[k + r * step] : 0.f;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (q[r] != 0.f && !charge_fits(q[r], e)) charge_small(A, P, Q, Qa, k + r * step);
+  }
 }
 
 // h + l = a running FP32 sum and its exact rounding errors (Knuth's two-sum)
@@ -940,7 +996,9 @@ void charge32(pic_ctx *c) {
   if (c->n_used == 0) return;
   using U = unsigned long long;
   // the flux accumulators are clear between steps: the first lends a plane
-  const ChargePlanes C{{(U *)c->Q, (U *)c->Qt}, {(U *)c->Qa, (U *)c->acc[0]}};
+  const ChargePlanes C{{(U *)c->Q, (U *)c->Qt}, {(U *)c->Qa, (U *)c->acc[0]},
+                       (long long *)c->scratch, (long long)(c->scratch_bytes / sizeof(long long))};
+  cudaMemsetAsync(c->d_cnt + CNT_SMALL, 0, sizeof(long long), c->stream);
   const Args32 A = make_args(c, 0.0);
   const unsigned blocks = (unsigned)ens_tile_blocks(c);
   if (c->tiles.TI == 8) ++c->launches, k_charge_tiles<8, 32><<<blocks, NT, 0, c->stream>>>(A, c->p32, C);
@@ -949,6 +1007,7 @@ void charge32(pic_ctx *c) {
   const Grid &G = c->G;
   const dim3 gr((G.nth + 1 + 31) / 32, (G.nr + 2 * G.g + 1 + 7) / 8);
   ++c->launches, k_charge_finish<<<gr, dim3(32, 8), 0, c->stream>>>(G, c->qexp, C, (U *)c->acc[0], c->Q, c->Qa);
+  ++c->launches, k_charge_small<<<4 * 152, 256, 0, c->stream>>>(A, c->p32, C, c->Q, c->Qa);
 }
 
 void reduce_particles32(pic_ctx *c) {
