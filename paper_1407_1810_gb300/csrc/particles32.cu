@@ -507,12 +507,21 @@ __device__ __forceinline__ void two_sum(float v, float &h, float &l) {
   h = s;
 }
 
+// whether the largest of eight magnitudes leaves the error-carrying sum of the
+// eight its range: no overflow, and what falls below the normal numbers is below
+// 2^-53 of it
+__device__ __forceinline__ bool sums_in_range(float m) {
+  const unsigned b = __float_as_uint(m), lo = (127 - 70) << 23, hi = (127 + 120) << 23;
+  return b == 0 || b - lo <= hi - lo;
+}
+
 // Kinetic energy, charge and live count.  Each particle's (gamma - 1) |qw| is
 // formed in FP32 (gamma - 1 = u^2 / (1 + gamma): no cancellation) and summed
 // in FP64 eight at a time, the eight through an error-carrying FP32 sum: a
 // conversion and an addition on the FP64 pipe per particle and sum kept this
 // pass FP64-bound (5e7 particles, 0.8 GB: 0.40 ms; 0.26 four, 0.24 eight at a
-// time, 0.18 with the eight's loads issued together).
+// time, 0.18 with the eight's loads issued together).  Eight next to an end of
+// FP32's range (charges up to 2^100 are accepted) are added in FP64.
 __global__ void k_reduce32(Parts32 P, int64_t n, double qm, double *acc, long long *live) {
   double kin = 0.0, ch = 0.0;
   long long l = 0;
@@ -527,17 +536,31 @@ __global__ void k_reduce32(Parts32 P, int64_t n, double qm, double *acc, long lo
       q[r] = P.qw[y]; a[r] = P.ur[y]; b[r] = P.ut[y]; c[r] = P.up[y];
       if (x >= n) q[r] = 0.f;
     }
-    float kh = 0.f, kl = 0.f, qh = 0.f, ql = 0.f;
+    float e[8], em = 0.f, qm8 = 0.f;
     int m = 0;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const float u2 = a[r] * a[r] + b[r] * b[r] + c[r] * c[r], e = fabsf(q[r]) * (u2 / (1.f + sqrtf(1.f + u2)));
-      two_sum(q[r] != 0.f ? e : 0.f, kh, kl);
-      two_sum(q[r], qh, ql);
+      const float u2 = a[r] * a[r] + b[r] * b[r] + c[r] * c[r], w = fabsf(q[r]) * (u2 / (1.f + sqrtf(1.f + u2)));
+      e[r] = q[r] != 0.f ? w : 0.f;
+      em = fmaxf(em, e[r]);
+      qm8 = fmaxf(qm8, fabsf(q[r]));
       m += q[r] != 0.f;
     }
-    kin += (double)kh + (double)kl;
-    ch += (double)qh + (double)ql;
+    if (sums_in_range(em) && sums_in_range(qm8)) {
+      float kh = 0.f, kl = 0.f, qh = 0.f, ql = 0.f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        two_sum(e[r], kh, kl);
+        two_sum(q[r], qh, ql);
+      }
+      kin += (double)kh + (double)kl;
+      ch += (double)qh + (double)ql;
+    } else {
+      for (int r = 0; r < 8; ++r) {
+        kin += e[r];
+        ch += q[r];
+      }
+    }
     l += m;
   }
   block_sum3(kin / qm, ch, l, acc + ACC_KIN, acc + ACC_CHARGE, live);
