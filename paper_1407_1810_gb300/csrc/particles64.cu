@@ -319,7 +319,9 @@ __global__ void __launch_bounds__(256) k_particles64(const __grid_constant__ Arg
   else D1 = m * recip64(ir) * A.inv_dxi;
   const double Px = fma(a, st, fma(b, ct, st)), Pz = fma(a, ct, fma(-b, st, ct));  // before rotating back
   const double R2 = fma(Px, Px, c * c);
-  const bool off = hi_word(R2) != 0, back = hi_word(Px) < 0;  // off the axis; across it
+  // off the axis by more than rounds to nothing (a square below the normal
+  // numbers: Px, c, u_th and u_ph all under 1e-150); across it
+  const bool off = hi_word(R2) >= 0x00100000, back = hi_word(Px) < 0;
   const double iR = off ? rsqrt64(R2) : 0.0, R = R2 * iR;
   const double stn = R * inv_rn, ctn = Pz * inv_rn;
   double D2;
@@ -333,7 +335,7 @@ __global__ void __launch_bounds__(256) k_particles64(const __grid_constant__ Arg
   }
   // azimuth swept, and the momentum in the new local frame
   const double cp = off ? Px * iR : 1.0, sp = off ? c * iR : 0.0;
-  double phi = !back && (hi_word(sp) & 0x7fffffff) < 0x3fc00000 ? asin_series64(sp) : atan2(c, Px);
+  double phi = !back && off && (hi_word(sp) & 0x7fffffff) < 0x3fc00000 ? asin_series64(sp) : atan2(c, Px);
   const double ux = fma(u[0], st, u[1] * ct), uz = fma(u[0], ct, -(u[1] * st));
   if (back) {  // rare: see AxisTies
     const double w2 = u[2] * u[2];
