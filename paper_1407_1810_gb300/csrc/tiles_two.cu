@@ -570,21 +570,27 @@ __device__ __forceinline__ void step32(const Args32 &A, const W &w, float fs, in
   }
   // displaced point, (R, z) before rotating back; kap = R' - Px
   const V Px = fma_(a, st, fma_(b, ct, st)), Pz = sub_(fma_(a, ct, ct), mul_(b, st));
-  const V R2 = fma_(Px, Px, fma_(c, c, 1e-30f));  // (the constant: no 0 / 0 on the axis)
+  const V R2 = fma_(Px, Px, fma_(c, c, 2e-38f));  // (the constant, a normal number: no 0 / 0 on the axis)
   const V iRn = rsqrt_(R2), Rn = mul_(R2, iRn);
   V kap = mul_(c2, rcp_(fma_(R2, iRn, Px)));
   const V sph = mul_(c, iRn);        // sine of the azimuth swept
   V phi = asin_series(sph);
   {
-    bool far = false;  // across the axis, or turning by a large azimuth next to it
+    bool far = false;  // across the axis, on it, or turning by a large azimuth next to it
 #pragma unroll
-    for (int l = 0; l < NL; ++l) far |= !(Px[l] > 0.f && fabsf(sph[l]) < 0.25f);
+    for (int l = 0; l < NL; ++l) far |= !(Px[l] > 1e-17f && fabsf(sph[l]) < 0.25f);
     if (far) {
 #pragma unroll
       for (int l = 0; l < NL; ++l)
-        if (on[l] && !(Px[l] > 0.f && fabsf(sph[l]) < 0.25f)) {
-          if (!(Px[l] > 0.f)) kap[l] = Px[l] < 0.f ? __fsub_rn(Rn[l], Px[l]) : (R2[l] > 1.1e-30f ? Rn[l] : 0.f);
-          phi[l] = azimuth(c[l], Px[l], Rn[l]);
+        if (on[l] && !(Px[l] > 1e-17f && fabsf(sph[l]) < 0.25f)) {
+          if (!(Px[l] > 0.f)) kap[l] = Px[l] < 0.f ? __fsub_rn(Rn[l], Px[l]) : (R2[l] > 2.2e-38f ? Rn[l] : 0.f);
+          float x = Px[l], y = c[l], R = Rn[l];
+          if (R2[l] < 1e-20f) {  // lengths whose squares lose bits: 2^60 times them
+            x = __fmul_rn(x, 0x1p60f);
+            y = __fmul_rn(y, 0x1p60f);
+            R = sqrtf(__fmaf_rn(x, x, __fmul_rn(y, y)));
+          }
+          phi[l] = azimuth(y, x, R);
           if (Px[l] < 0.f && p[2][l] * p[2][l] <= (float)(AXIS_TIE * AXIS_TIE) *
                                                        (p[0][l] * p[0][l] + p[1][l] * p[1][l] + p[2][l] * p[2][l]))
             phi[l] = axis_tie(A.ties, A.ids[k0 + l], phi[l]);  // rare: see AxisTies
