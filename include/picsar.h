@@ -245,9 +245,10 @@ int pic_set_clock(pic_ctx *c, int64_t step, int64_t next_id);
 
 /* Per-kernel timing of later steps with CUDA events on the context's stream:
  * enable = 1 starts accumulating; pic_get_profile writes the mean milliseconds
- * per launch of [particle kernel, 0, 0, grid update, injection, sort] into ms6
- * and the number of timed steps into *steps.  The grid update holds the filter
- * and both Yee kernels (slots 1 and 2 timed kernels that are part of it). */
+ * per launch of [particle kernel, flux conversion, filter, grid update,
+ * injection, sort] into ms6 and the number of timed steps into *steps.  Up to
+ * four filter passes, and the conversion with them, are part of the grid update's
+ * first kernel: slots 1 and 2 are then 0 (slot 1 always on the FP64 path). */
 int pic_profile(pic_ctx *c, int32_t enable);
 int pic_get_profile(pic_ctx *c, double *ms6, int64_t *steps);
 

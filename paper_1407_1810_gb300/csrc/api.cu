@@ -819,6 +819,16 @@ void pic_step_body(pic_ctx *c) {
   if (c->d.precision == PIC_FP64) particles64(c, t);
   else particles32(c, t);
   prof_end(c, pr);
+  if (filter_apart(c)) {
+    if (c->d.precision == PIC_FP32) {
+      pr = prof_begin(c, PROF_REDUCE);
+      fields_flux(c);
+      prof_end(c, pr);
+    }
+    pr = prof_begin(c, PROF_FILTER);
+    fields_filter(c);
+    prof_end(c, pr);
+  }
   pr = prof_begin(c, PROF_FIELDS);
   fields_e_step(c);
   fields_b_step(c, true);

@@ -918,21 +918,31 @@ void fields_b_start(pic_ctx *c) {
   c->bh_ok = true;
 }
 
+bool filter_apart(const pic_ctx *c) { return c->d.n_filt > FUSE_FILT; }
+
+void fields_flux(pic_ctx *c) {
+  EnsFieldArg a;
+  ens_fill_field_arg(c, &a);
+  const Grid &G = c->G;
+  ++c->launches, launch_on(c->stream, c->overlap, k_flux_from_acc, grid2(G.nr + 2 * G.g + 1, G.nth + 1), dim3(BX, BY), a);
+}
+
+void fields_filter(pic_ctx *c) {
+  EnsFieldArg a;
+  ens_fill_field_arg(c, &a);
+  const Grid &G = c->G;
+  const dim3 gr = grid2(G.nr + 2 * G.g + 1, G.nth + 1);
+  for (int p = 0; p < c->d.n_filt; ++p)
+    for (int k = 0; k < 3; ++k)
+      ++c->launches, launch_on(c->stream, c->overlap, k_filter, gr, dim3(BX, BY), G, (p & 1) ? a.Ftmp[k] : a.Fin[k],
+                               (p & 1) ? a.Fin[k] : a.Ftmp[k], k == 1);
+}
+
 void fields_e_step(pic_ctx *c) {
   EnsFieldArg a;
   ens_fill_field_arg(c, &a);
-  const bool fp32 = c->d.precision == PIC_FP32;
-  if (c->d.n_filt > FUSE_FILT) {
-    const Grid &G = c->G;
-    const dim3 gr = grid2(G.nr + 2 * G.g + 1, G.nth + 1);
-    if (fp32) ++c->launches, launch_on(c->stream, c->overlap, k_flux_from_acc, gr, dim3(BX, BY), a);
-    for (int p = 0; p < c->d.n_filt; ++p)
-      for (int k = 0; k < 3; ++k)
-        ++c->launches, launch_on(c->stream, c->overlap, k_filter, gr, dim3(BX, BY), G, (p & 1) ? a.Ftmp[k] : a.Fin[k],
-                                                                    (p & 1) ? a.Fin[k] : a.Ftmp[k], k == 1);
-  }
   const unsigned nb = (unsigned)ens_blocks(c, ENS_BAND);
-  if (fp32) ++c->launches, launch_on(c->stream, c->overlap, k_e_step<true>, nb, dim3(BX, BY), a);
+  if (c->d.precision == PIC_FP32) ++c->launches, launch_on(c->stream, c->overlap, k_e_step<true>, nb, dim3(BX, BY), a);
   else ++c->launches, launch_on(c->stream, c->overlap, k_e_step<false>, nb, dim3(BX, BY), a);
 }
 

@@ -204,6 +204,9 @@ namespace pic {
 // fields.cu
 int lossy_first_row(const pic_ctx *c);  // -1: no lossy layer
 void fields_b_start(pic_ctx *c);       // bh of the stored fields, when it does not match them
+bool filter_apart(const pic_ctx *c);   // more passes than the E update takes: before it, fields_flux (FP32) and fields_filter
+void fields_flux(pic_ctx *c);          // FP32: the deposit to FP64
+void fields_filter(pic_ctx *c);        // the filter pass by pass
 void fields_e_step(pic_ctx *c);        // filtered flux of the deposit, E update, lossy layer on E
 void fields_b_step(pic_ctx *c, bool sigma);  // B update, lossy layer, ghosts, FP32 copies; clears the deposit;
                                              // sigma: the injection's surface charge at the step's end

@@ -393,7 +393,13 @@ int slab_step(pic_slabs *g) {
         if ((e = halo_sum(g, g->ctx[s], g->ctx[s + 1], g->ctx[s]->Ft[k], g->ctx[s + 1]->Ft[k]))) return e;
   }
   static const int B3[3] = {BR, BTH, BPH}, E3[3] = {ER, ETH, EPH};
-  for (pic_ctx *c : g->ctx) fields_e_step(c);
+  for (pic_ctx *c : g->ctx) {
+    if (filter_apart(c)) {
+      if (c->d.precision == PIC_FP32) fields_flux(c);
+      fields_filter(c);
+    }
+    fields_e_step(c);
+  }
   if ((e = exchange_fields(g, E3, 3))) return e;
   for (pic_ctx *c : g->ctx) fields_b_step(c, false);
   if ((e = exchange_fields(g, E3, 3)) || (e = exchange_fields(g, B3, 3))) return e;  // with the axis ghosts
