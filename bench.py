@@ -159,16 +159,28 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
+# what the tile kernel's traffic depends on: the kernel, its window and unit
+# ranges, and the sort that orders and cuts its particles
+TRAFFIC_SOURCES = ["tiles_two.cu", "tiles32.cuh", "particles32.cu"]
+
+
+def traffic_hash():
+    h = hashlib.sha256()
+    for f in TRAFFIC_SOURCES:
+        with open(os.path.join(ROOT, "paper_1407_1810_gb300", "csrc", f), "rb") as s:
+            h.update(s.read())
+    return h.hexdigest()[:16]
+
+
 def recorded_traffic():
     """DRAM bytes per particle of the tile kernel from the committed ncu
-    summary, if the kernel source has not changed since it was taken."""
+    summary, if none of the sources it depends on has changed since it was
+    taken."""
     p = os.path.join(ROOT, "profiles", "k_tiles32_traffic.json")
-    src = os.path.join(ROOT, "paper_1407_1810_gb300", "csrc", "tiles_two.cu")
     if not os.path.exists(p):
         return None
     d = json.load(open(p))
-    h = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-    if d.get("source_sha256_16") != h:
+    if d.get("source_sha256_16") != traffic_hash():
         return None
     return float(d["dram_bytes_per_particle"])
 
