@@ -126,14 +126,14 @@ struct Block {
 };
 
 // ---- metric tables ----------------------------------------------------------
-constexpr int METRIC_ROWS = 21, METRIC_COLS = 18;  // row and column tables
+constexpr int METRIC_ROWS = 17, METRIC_COLS = 15;  // row and column tables
 std::vector<double> build_metric(const pic_ctx *c) {
   const pic_desc &d = c->d;
   const Grid &G = c->G;
   const int NRr = d.nr + 2 * G.PI + 1, NC = G.LD;
   const int nrg = G.nr_glob;  // rows of the whole grid (a slab's tables hold its global rows)
-  // row tables 0-12 (geometry) and 13-20 (update coefficients); column
-  // tables 0-11 and 17 (geometry) and 12-16 (update coefficients)
+  // row tables 0-8 (geometry) and 9-16 (update coefficients); column tables
+  // 0-8 and 14 (geometry) and 9-13 (update coefficients)
   const int nrow = METRIC_ROWS, ncol = METRIC_COLS;
   const double hh = 0.5 * G.dt, dt = G.dt;
   std::vector<double> h((size_t)nrow * NRr + (size_t)ncol * NC, 0.0);
@@ -147,27 +147,23 @@ std::vector<double> build_metric(const pic_ctx *c) {
     row(0)[ii] = rn;
     row(1)[ii] = rh;
     row(2)[ii] = 1.0 / rn;
-    row(3)[ii] = 2.0 / (rn1 * rn1 - rn * rn);
-    row(4)[ii] = rn1 - rn;
-    row(5)[ii] = 1.0 / rh;
-    row(6)[ii] = 1.0 / (2.0 * M_PI * rh * rh);
-    row(7)[ii] = 2.0 / (rh * rh - rhm * rhm);
-    row(8)[ii] = rh - rhm;
-    row(9)[ii] = 1.0 - sigma_star(d, i, nrg);
-    row(10)[ii] = 1.0 - sigma_star(d, i + 0.5, nrg);
+    row(3)[ii] = 1.0 / (2.0 * M_PI * rh * rh);
+    row(4)[ii] = 2.0 / (rh * rh - rhm * rhm);
+    row(5)[ii] = 1.0 - sigma_star(d, i, nrg);
+    row(6)[ii] = 1.0 - sigma_star(d, i + 0.5, nrg);
     const double id2n = 2.0 / (rn1 * rn1 - rn * rn);
-    row(13)[ii] = hh / rn;
-    row(14)[ii] = hh * id2n * rn;
-    row(15)[ii] = hh * id2n * rn1;
-    row(16)[ii] = hh * id2n * (rn1 - rn);
-    row(17)[ii] = dt / rh;
-    row(18)[ii] = dt * rhm;
-    row(19)[ii] = dt * rh;
-    row(20)[ii] = dt * (rh - rhm);
+    row(9)[ii] = hh / rn;
+    row(10)[ii] = hh * id2n * rn;
+    row(11)[ii] = hh * id2n * rn1;
+    row(12)[ii] = hh * id2n * (rn1 - rn);
+    row(13)[ii] = dt / rh;
+    row(14)[ii] = dt * rhm;
+    row(15)[ii] = dt * rh;
+    row(16)[ii] = dt * (rh - rhm);
     if (i >= 0 && i <= nrg) {
       double a = std::fmax(i - 0.5, 0.0), b = std::fmin(i + 0.5, (double)nrg);
-      row(11)[ii] = 2.0 * M_PI / 3.0 * (std::pow(fr(b), 3) - std::pow(fr(a), 3));
-      row(12)[ii] = i < nrg ? 2.0 * M_PI / 3.0 * (std::pow(rn1, 3) - std::pow(rn, 3)) : 0.0;
+      row(7)[ii] = 2.0 * M_PI / 3.0 * (std::pow(fr(b), 3) - std::pow(fr(a), 3));
+      row(8)[ii] = i < nrg ? 2.0 * M_PI / 3.0 * (std::pow(rn1, 3) - std::pow(rn, 3)) : 0.0;
     }
   }
   auto th = [&](double x) { return h_fth(d, x); };
@@ -177,30 +173,29 @@ std::vector<double> build_metric(const pic_ctx *c) {
     if (j >= 0 && j <= d.nth) {
       col(0)[cc] = std::sin(th(j));
       col(1)[cc] = std::cos(th(j));
-      col(9)[cc] = 1.0 / (ctb(j - 1) - ctb(j));
-      col(10)[cc] = std::cos(th(std::fmax(j - 0.5, 0.0))) - std::cos(th(std::fmin(j + 0.5, (double)d.nth)));
+      col(6)[cc] = 1.0 / (ctb(j - 1) - ctb(j));
+      col(7)[cc] = std::cos(th(std::fmax(j - 0.5, 0.0))) - std::cos(th(std::fmin(j + 0.5, (double)d.nth)));
     }
     if (j >= 0 && j < d.nth) {
       col(2)[cc] = 1.0 / (std::cos(th(j)) - std::cos(th(j + 1)));
       col(3)[cc] = 1.0 / (th(j + 1) - th(j));
       col(4)[cc] = std::sin(th(j + 0.5));
-      col(5)[cc] = 1.0 / std::sin(th(j + 0.5));
-      col(11)[cc] = std::cos(th(j)) - std::cos(th(j + 1));
-      col(17)[cc] = std::cos(th(j + 0.5));
+      col(8)[cc] = std::cos(th(j)) - std::cos(th(j + 1));
+      col(14)[cc] = std::cos(th(j + 0.5));
     }
-    if (j >= 1 && j < d.nth) col(6)[cc] = 1.0 / (th(j + 0.5) - th(j - 0.5));
+    if (j >= 1 && j < d.nth) col(5)[cc] = 1.0 / (th(j + 0.5) - th(j - 0.5));
   }
   for (int cc = 0; cc < NC; ++cc) {  // products of the geometry columns (zero where a factor is)
     const int j = cc - G.PJ;
     const double stb = j >= 0 && j < d.nth ? col(4)[cc] : 0.0, stbm = cc >= 1 && j >= 1 && j <= d.nth ? col(4)[cc - 1] : 0.0;
     if (j >= 0 && j < d.nth) {
-      col(12)[cc] = col(0)[cc] * col(2)[cc];
-      col(13)[cc] = col(0)[cc + 1] * col(2)[cc];
-      col(16)[cc] = col(5)[cc] * (0.5 / M_PI);
+      col(9)[cc] = col(0)[cc] * col(2)[cc];
+      col(10)[cc] = col(0)[cc + 1] * col(2)[cc];
+      col(13)[cc] = 1.0 / std::sin(th(j + 0.5)) * (0.5 / M_PI);
     }
     if (j >= 0 && j <= d.nth) {
-      col(14)[cc] = stb * col(9)[cc];
-      col(15)[cc] = stbm * col(9)[cc];
+      col(11)[cc] = stb * col(6)[cc];
+      col(12)[cc] = stbm * col(6)[cc];
     }
   }
   return h;
@@ -214,16 +209,16 @@ void metric_pointers(pic_ctx *c) {
   auto dr = [&](int t) { return R + (size_t)t * NRr; };
   auto dc = [&](int t) { return C + (size_t)t * NC; };
   Metric &m = G.m;
-  m.r_n = dr(0); m.r_h = dr(1); m.inv_r_n = dr(2); m.inv_dr2_n = dr(3); m.dr_n = dr(4);
-  m.inv_r_h = dr(5); m.inv_area_h = dr(6); m.inv_dr2_h = dr(7); m.dr_h = dr(8);
-  m.keep_n = dr(9); m.keep_h = dr(10); m.vol_r_n = dr(11); m.vol_r_h = dr(12);
+  m.r_n = dr(0); m.r_h = dr(1); m.inv_r_n = dr(2);
+  m.inv_area_h = dr(3); m.inv_dr2_h = dr(4);
+  m.keep_n = dr(5); m.keep_h = dr(6); m.vol_r_n = dr(7); m.vol_r_h = dr(8);
   m.sin_t = dc(0); m.cos_t = dc(1); m.inv_dcos_t = dc(2); m.inv_dth_t = dc(3);
-  m.sin_tb = dc(4); m.inv_sin_tb = dc(5); m.inv_dtb = dc(6);
-  m.inv_dcos_tb = dc(9); m.vol_t_n = dc(10); m.vol_t_h = dc(11);
-  m.bR = dr(13); m.bT0 = dr(14); m.bT1 = dr(15); m.bP = dr(16);
-  m.eR = dr(17); m.w0 = dr(18); m.w1 = dr(19); m.wd = dr(20);
-  m.cB1 = dc(12); m.cB2 = dc(13); m.cE1 = dc(14); m.cE2 = dc(15); m.cF = dc(16);
-  m.cos_tb = dc(17);
+  m.sin_tb = dc(4); m.inv_dtb = dc(5);
+  m.inv_dcos_tb = dc(6); m.vol_t_n = dc(7); m.vol_t_h = dc(8);
+  m.bR = dr(9); m.bT0 = dr(10); m.bT1 = dr(11); m.bP = dr(12);
+  m.eR = dr(13); m.w0 = dr(14); m.w1 = dr(15); m.wd = dr(16);
+  m.cB1 = dc(9); m.cB2 = dc(10); m.cE1 = dc(11); m.cE2 = dc(12); m.cF = dc(13);
+  m.cos_tb = dc(14);
 }
 
 // ---- particle buffers ----------------------------------------------------------

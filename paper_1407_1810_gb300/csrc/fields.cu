@@ -876,7 +876,6 @@ void ens_fill_field_arg(const pic_ctx *c, EnsFieldArg *a) {
     a->Fout[k] = fused ? c->F[k] : ((c->d.n_filt & 1) ? a->Ftmp[k] : a->Fin[k]);
     a->acc[k] = c->acc[k];
   }
-  a->grid_elems = c->grid_elems;
   a->cnt = c->d_cnt;
   a->qexp = c->qexp;
   a->sig = c->sig;

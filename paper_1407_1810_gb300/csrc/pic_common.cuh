@@ -58,12 +58,8 @@ enum ErrBits { ERR_COURANT = 1, ERR_CAPACITY = 2, ERR_NAN = 4, ERR_RANGE = 8, ER
 struct Metric {
   const double *r_n, *r_h;          // f_r(i), f_r(i + 1/2)
   const double *inv_r_n;            // 1 / r_i
-  const double *inv_dr2_n;          // 2 / (r_{i+1}^2 - r_i^2)
-  const double *dr_n;               // r_{i+1} - r_i
-  const double *inv_r_h;            // 1 / rb_i
   const double *inv_area_h;         // 1 / (2 pi rb_i^2)
   const double *inv_dr2_h;          // 2 / (rb_i^2 - rb_{i-1}^2)
-  const double *dr_h;               // rb_i - rb_{i-1}
   const double *keep_n, *keep_h;    // 1 - sigma*(i), 1 - sigma*(i + 1/2)  (Eq. EBcond)
   const double *vol_r_n, *vol_r_h;  // radial factors of the cell volumes (energy)
   const double *sin_t;              // sin th_j
@@ -72,7 +68,6 @@ struct Metric {
   const double *inv_dth_t;          // 1 / (th_{j+1} - th_j)
   const double *sin_tb;             // sin tb_j, with sin tb_{-1} = sin tb_{nth} = 0
   const double *cos_tb;             // cos tb_j (j < nth)
-  const double *inv_sin_tb;         // 1 / sin tb_j
   const double *inv_dcos_tb;        // 1 / (cos tb_{j-1} - cos tb_j), caps at j = 0, nth
   const double *inv_dtb;            // 1 / (tb_j - tb_{j-1})
   const double *vol_t_n, *vol_t_h;  // meridional factors of the cell volumes

@@ -115,7 +115,6 @@ struct EnsFieldArg {
   double *Fin[3], *Ftmp[3], *Fout[3];  // FP64 deposit; scratch of the pass-by-pass filter; filtered flux
   float *f32[6];
   long long *acc[3];
-  size_t grid_elems;
   long long *cnt;
   long long *qexp;                     // the fixed-point exponent counter
   double *sig;                         // two buffers of nth + 1
