@@ -689,12 +689,13 @@ int pic_create_context(pic_ctx **out, const pic_desc &d, void *stream, int i0, i
     }
     // The grid bounds the arguments of the move's series: dx dxi <= dxi for
     // exp; with eps = dt / r(-g) (speed < c) the relative displacement s <=
-    // 2 eps + 3 eps^2 for log1p and the turning angle below eps for atan and
-    // the sin / cos series.  With dxi <= 1/16 and eps <= 1/40 every series'
-    // relative truncation stays below 2^-28, 1/16 of an FP32 ulp (at the
-    // bounds, evaluated in FP64: exp 8.8e-11, log1p 2.9e-9, atan and the
-    // sin / cos series below 1e-13), so the step uses the series without
-    // the general fallback
+    // 2 eps + 3 eps^2 for log1p and (1 + s)^-1/2, and the turning angle's sine
+    // below eps / (1 - eps) for the arcsine (the one-particle form: the angle's
+    // arctangent, sine and cosine).  With dxi <= 1/16 and eps <= 1/40 every
+    // series' relative truncation stays below 2^-28, 1/16 of an FP32 ulp (at the
+    // bounds: exp 8.8e-11, log1p 2.9e-9, (1 + s)^-1/2 2.2e-10, the turn's arcsine
+    // and cosine below 3e-11, the one-particle form's below 1e-13), so the step
+    // uses the series without the general fallback
     c->small_steps = d.r_map == PIC_R_LOG && G.dxi <= 1.0 / 16 && G.dt / h_fr(d, G.dxi, -G.g) <= 1.0 / 40;
     if ((e = upload(c->th_n32, tf.data(), tf.size() * sizeof(float2))) ||
         (e = upload(c->r_n32, rn.data(), nrp * sizeof(float))) ||

@@ -1,20 +1,10 @@
-// particles32.cu -- the FP32 cell+offset particle path (the hot path):
-//
-//  * particles are kept binned by tiles of TI x TJ cells (counting sort by tile,
-//    every sort_interval steps; deleted particles are dropped by the sort);
-//  * one CTA per tile stages a window of the FP32 field copies (tile + halo H
-//    + the stencil) in shared memory, gathers, pushes and moves every particle
-//    of its bin, and deposits the Villasenor-Buneman fluxes into shared-memory
-//    int64 fixed-point accumulators (exact and order independent), flushed
-//    with one global atomic per nonzero window node;
-//  * a particle that drifted out of its tile's window since the last sort, or
-//    was injected after it, takes the same code with global-memory accessors.
-//
-// Position = integer cell + FP32 offset in [0, 1).  The move runs in the
-// particle's local frame: the radial increment comes from log1p of the
-// relative displacement, the meridional one from the exact rotation angle of
-// the displaced point, so an offset keeps ~1e-7 cell accuracy anywhere on the
-// grid instead of the ~1e-4 cell an absolute FP32 r or theta would give.
+// particles32.cu -- the FP32 cell+offset particle path (the hot path) around its
+// tile kernel (tiles_one.cu, tiles_two.cu): the particles are kept binned by tiles
+// of TI x TJ cells (counting sort every sort_interval steps, which drops the
+// deleted ones), each tile's bin is cut into work units, one CTA each, and a step
+// launches the tile kernel's form for the grid over them.  Also: the node charge
+// and the particle sums of the diagnostics, the batched launches and the batched
+// sort of ensemble members.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -574,11 +564,14 @@ constexpr int TRW_WARP = 32;
 // 1e8 49.6 and 36.9; a whole run of 448 x 416: 8.05 and 7.38); on a small grid,
 // bound by latency and by the grid phase, the two are closer (72 x 56 rotator
 // 0.65 and 0.67 ms, 192 x 160 dipole 1.35 and 1.27, 250 x 231 monopole 1.51 and
-// 1.41; 64-member ensemble, 40 steps: 49.1 and 46.8).  They round differently,
-// and the sparse plasmas run on small grids (ensemble members of a few particles
-// a cell) amplify a rounding a hundredfold in eighty steps: those keep the form
-// and the bits they had.  The grid alone decides, so that a member, a slab and a
-// run of its own agree.
+// 1.41; 64-member ensemble, 40 steps: 49.1 and 46.8).  They round differently and
+// neither is the less exact: against the FP64 path, over 78 runs of sparse plasmas
+// (2000 to 60000 particles, grids on both sides of the line, six seeds each, 1 to
+// 80 steps), the two-particle form's momenta are off by 0.5 to 1.07 times as
+// much as the other's, its positions by 0.69 to 1.03, its fields by as much one
+// way as the other.  The line is the largest grid of an ensemble's members (256 x
+// 512): up to it results keep the bits of the one-particle form.  The grid alone
+// decides, so that a member, a slab and a run of its own agree.
 constexpr int64_t PACK_CELLS = 1 << 17;
 bool use_packed(const pic_ctx *c) { return (int64_t)c->G.nr_glob * c->G.nth > PACK_CELLS; }
 

@@ -21,11 +21,12 @@ namespace pic {
 // launch: a kernel is set up while the one before it runs, and this call, before
 // anything it reads or writes, waits until that kernel has ended and its results
 // are visible.  Launched without the attribute (launch_on, overlap false) the
-// call has no effect.  No kernel lets its dependents start before it ends
-// (griddepcontrol.launch_dependents): blocks that wait beside a particle kernel
-// cost it more than they gain (64 x 64 FP64 step 101 us without overlap, 123
-// with the early start, 91 so; 72 x 56 FP32 40.6, 34.7, 30.5; 192 x 160 56.2,
-// 56.7, 46; 250 x 231 84, -, 75).
+// call has no effect.  No kernel of a single context's step lets its dependents
+// start before it ends (griddepcontrol.launch_dependents): blocks that wait beside
+// a particle kernel cost it more than they gain (64 x 64 FP64 step 101 us without
+// overlap, 123 with the early start, 91 so; 72 x 56 FP32 40.6, 34.7, 30.5; 192 x
+// 160 56.2, 56.7, 46; 250 x 231 84, -, 75).  The tile launches of an ensemble's
+// step do, for each other (ens_tiles32).
 __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void follow() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -110,7 +111,8 @@ constexpr double PI_D = 3.14159265358979323846;
 // (double)v * 2^s built on the integer pipes: v rounded to 53 bits (to
 // nearest, ties to even, as the FP64 conversion does; exact for the sums
 // below 2^53 that occur in practice) and the power of two added to the
-// exponent, which is exact while the result stays normal (s in [-126, 64] here).
+// exponent, which is exact while the result stays normal (s in [-149, 64] here:
+// the charge exponent, -90 to 100, less 36 and four bits a filter pass, or 59).
 // The same IEEE value as the conversion and multiply, without the FP64 pipe,
 // whose rate on this part made the conversion pass compute-bound.
 __device__ inline double fixed_to_f64(long long v, int s) {
