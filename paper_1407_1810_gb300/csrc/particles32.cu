@@ -802,10 +802,11 @@ static int64_t unit_size(const pic_ctx *c) {
   int64_t unit = NT;
   for (int64_t m = 1; m <= 64 || m * tiles <= 4 * SLOTS; ++m) {
     const double share = avg / m;
+    const int64_t u = std::max<int64_t>(NT, (int64_t)(1.1 * share) + 1);
     const double cost = std::ceil((double)m * tiles / SLOTS) * (std::ceil(share / NT) + 1.5);
-    if (cost < best) {
+    if (u <= room && cost < best) {
       best = cost;
-      unit = std::max<int64_t>(NT, (int64_t)(1.1 * share) + 1);
+      unit = u;
     }
     if (share <= NT) break;
   }
