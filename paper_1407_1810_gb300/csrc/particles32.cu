@@ -331,7 +331,8 @@ constexpr int QRANGE = 5;
 constexpr int QFLUSH = (1 << 12) / NT;               // passes of NT particles: 2^12 terms of less than 2^20
 struct ChargePlanes {
   unsigned long long *hi[2], *lo[2];  // sums of the high and the low QSPLIT bits, of positive and negative charge
-  long long *list, cap;               // the slots of the first cap charges below 2^(e - QRANGE) (CNT_SMALL counts all)
+  long long *list, cap;               // the slots of the first cap charges below 2^(e - QRANGE)
+  long long *small, *next;            // all of them counted; the next call's counter, which this call clears
 };
 
 // w in [0, 1) as a fraction of 2^64 (exact from 2^-40 on)
@@ -352,9 +353,9 @@ __device__ __forceinline__ unsigned long long charge_units(float q, int e) {
 
 // particle k into the list of small charges (a list that has run over needs no
 // more of them)
-__device__ __forceinline__ void charge_list(const Args32 &A, const ChargePlanes &C, int64_t k) {
-  if (*(volatile long long *)(A.cnt + CNT_SMALL) > C.cap) return;
-  const long long at = (long long)atomicAdd((unsigned long long *)A.cnt + CNT_SMALL, 1ull);
+__device__ __forceinline__ void charge_list(const ChargePlanes &C, int64_t k) {
+  if (*(volatile long long *)C.small > C.cap) return;
+  const long long at = (long long)atomicAdd((unsigned long long *)C.small, 1ull);
   if (at < C.cap) C.list[at] = k;
 }
 
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(NT) k_charge_tiles(Args32 A, Parts32 P, Charge
       if (dy >= 1.f) { dy = 0.f; ++cj; }  // on the south axis
       const int sg = q < 0.f;
       const bool fits = charge_fits(q, e);
-      if (!fits) charge_list(A, C, k);
+      if (!fits) charge_list(C, k);
       const ChargeShare s = charge_share(fits ? charge_units(q, e) : 0ull, dx, dy);
       if (binned && ci >= i0 - H && ci < i0 + TI + H && cj >= j0 - H && cj < j0 + TJ + H + 1) {
         const int o = (ci - wi0) * WJ + (cj - wj0);
@@ -447,6 +448,8 @@ __global__ void __launch_bounds__(NT) k_charge_tiles(Args32 A, Parts32 P, Charge
 // borrowed from the flux accumulators is cleared again.
 __global__ void k_charge_finish(Grid G, const long long *qexp, ChargePlanes C, unsigned long long *borrowed,
                                 double *Q, double *Qa) {
+  follow();
+  if ((blockIdx.x | blockIdx.y | threadIdx.x | threadIdx.y) == 0) *C.next = 0;
   const int i = -G.g + (int)(blockIdx.y * 8 + threadIdx.y), j = blockIdx.x * 32 + threadIdx.x;
   if (i > G.nr + G.g || j > G.nth) return;
   const size_t o = gidx(G, i, j);
@@ -473,7 +476,8 @@ __device__ __forceinline__ void charge_small(const Args32 &A, const Parts32 &P, 
 }
 
 __global__ void k_charge_small(Args32 A, Parts32 P, ChargePlanes C, double *Q, double *Qa) {
-  const int64_t n = A.cnt[CNT_SMALL], step = (int64_t)gridDim.x * blockDim.x;
+  follow();
+  const int64_t n = *C.small, step = (int64_t)gridDim.x * blockDim.x;
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n <= C.cap) {
     for (; k < n; k += step) charge_small(A, P, Q, Qa, C.list[k]);
@@ -1014,8 +1018,9 @@ void charge32(pic_ctx *c) {
   using U = unsigned long long;
   // the flux accumulators are clear between steps: the first lends a plane
   const ChargePlanes C{{(U *)c->Q, (U *)c->Qt}, {(U *)c->Qa, (U *)c->acc[0]},
-                       (long long *)c->scratch, (long long)(c->scratch_bytes / sizeof(long long))};
-  cudaMemsetAsync(c->d_cnt + CNT_SMALL, 0, sizeof(long long), c->stream);
+                       (long long *)c->scratch, (long long)(c->scratch_bytes / sizeof(long long)),
+                       c->d_cnt + CNT_SMALL + c->charge_slot, c->d_cnt + CNT_SMALL + 1 - c->charge_slot};
+  c->charge_slot ^= 1;
   const Args32 A = make_args(c, 0.0);
   const unsigned blocks = (unsigned)ens_tile_blocks(c);
   if (c->tiles.TI == 8) ++c->launches, k_charge_tiles<8, 32><<<blocks, NT, 0, c->stream>>>(A, c->p32, C);
@@ -1023,8 +1028,9 @@ void charge32(pic_ctx *c) {
   else ++c->launches, k_charge_tiles<16, 16><<<blocks, NT, 0, c->stream>>>(A, c->p32, C);
   const Grid &G = c->G;
   const dim3 gr((G.nth + 1 + 31) / 32, (G.nr + 2 * G.g + 1 + 7) / 8);
-  ++c->launches, k_charge_finish<<<gr, dim3(32, 8), 0, c->stream>>>(G, c->qexp, C, (U *)c->acc[0], c->Q, c->Qa);
-  ++c->launches, k_charge_small<<<4 * 152, 256, 0, c->stream>>>(A, c->p32, C, c->Q, c->Qa);
+  // (never captured: its callers wait for the result)
+  ++c->launches, launch_on(c->stream, true, k_charge_finish, gr, dim3(32, 8), G, c->qexp, C, (U *)c->acc[0], c->Q, c->Qa);
+  ++c->launches, launch_on(c->stream, true, k_charge_small, 4 * 152, 256, A, c->p32, C, c->Q, c->Qa);
 }
 
 void reduce_particles32(pic_ctx *c) {

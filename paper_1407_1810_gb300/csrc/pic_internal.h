@@ -28,7 +28,7 @@ constexpr int CELL_BIAS = 1024;
 
 // device counters (one int64 array)
 enum Counter { CNT_DELETED = 0, CNT_INJECTED = 1, CNT_LIVE = 2, CNT_SMAX = 3, CNT_GMAX = 4,
-               CNT_QMAX = 5, CNT_SORTED = 6, CNT_QEXP = 7, CNT_CAPPED = 8, CNT_TIES = 9, CNT_SMALL = 10, CNT_N };
+               CNT_QMAX = 5, CNT_SORTED = 6, CNT_QEXP = 7, CNT_CAPPED = 8, CNT_TIES = 9, CNT_SMALL = 10, CNT_SMALL2, CNT_N };
 constexpr int64_t TIE_LOG = 1 << 16;  // axis-crossing ties logged per context
 
 // FP32 path fixed-point deposit.  One flux unit is 2^(e - KFIX) with e =
@@ -183,6 +183,7 @@ struct pic_ctx {
   int64_t nhint = 0;
   int64_t step = 0, next_id = 0;
   int64_t launches = 0;  // kernels launched by this context
+  int charge_slot = 0;   // FP32: which of the counters CNT_SMALL, CNT_SMALL2 the next node charge counts in
   int host_err = 0;
   int steps_since_sort = 0;
   bool need_sort = false;
