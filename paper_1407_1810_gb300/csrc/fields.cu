@@ -49,8 +49,9 @@ __device__ __forceinline__ void curl_e(const Metric &m, int ri, int cj, double e
 // from the same formula with sin(tb_{-1}) = sin(tb_{nth}) = 0 and the cap
 // areas in inv_dcos_tb), then the lossy layer (Eq. EBcond: times 1 - sigma*
 // at the component's own radial stagger), whose rows keep the E before it in
-// epre for the second half step of B.  E_th, E_ph stay 0 on the conductors
-// (i = 0, nr) and E_ph on the axis.
+// epre for the second half step of B.  E_th, E_ph on the conductors (i = 0, nr)
+// and E_ph on the axis are not updated: 0, or what pic_set_fields left there,
+// which the layer scales like the rest.
 __device__ __forceinline__ void e_node(const EnsFieldArg &S, int i, int j, double Fr, double Ft, double Fp) {
   const Grid &G = S.G;
   const Metric &m = G.m;
@@ -66,19 +67,26 @@ __device__ __forceinline__ void e_node(const EnsFieldArg &S, int i, int j, doubl
     if (lossy) { S.epre[0][l] = e; e = __dmul_rn(e, m.keep_h[ri]); }
     S.f[ER][o] = e;
   }
-  // E_th, E_ph stay 0 on a conductor; a slab's open side is an interior row
+  // (a slab's open side is an interior row)
   const bool in = (i >= 1 || G.open_lo) && (i < G.nr || G.open_hi);
   const double w0 = m.w0[ri], w1 = m.w1[ri], id2 = m.inv_dr2_h[ri];
-  if (in && j < G.nth) {  // E_th at (i, j+1/2)
-    const double c = __fma_rn(-m.cF[cj], Ft, __fma_rn(w0, Bp[o - G.LD], -__dmul_rn(w1, Bp[o])));
-    double e = __fma_rn(id2, c, S.f[ETH][o]);
+  if ((in || lossy) && j < G.nth) {  // E_th at (i, j+1/2)
+    double e = S.f[ETH][o];
+    if (in) {
+      const double c = __fma_rn(-m.cF[cj], Ft, __fma_rn(w0, Bp[o - G.LD], -__dmul_rn(w1, Bp[o])));
+      e = __fma_rn(id2, c, e);
+    }
     if (lossy) { S.epre[1][l] = e; e = __dmul_rn(e, m.keep_n[ri]); }
     S.f[ETH][o] = e;
   }
-  if (in && j >= 1 && j < G.nth) {  // E_ph at (i, j)
-    const double c = __fma_rn(m.wd[ri], __dsub_rn(Br[o], Br[o - 1]), Fp);
-    const double k = __fma_rn(-m.inv_dtb[cj], c, __fma_rn(w1, Bt[o], -__dmul_rn(w0, Bt[o - G.LD])));
-    double e = __fma_rn(id2, k, S.f[EPH][o]);
+  const bool ph = in && j >= 1 && j < G.nth;
+  if (ph || lossy) {  // E_ph at (i, j)
+    double e = S.f[EPH][o];
+    if (ph) {
+      const double c = __fma_rn(m.wd[ri], __dsub_rn(Br[o], Br[o - 1]), Fp);
+      const double k = __fma_rn(-m.inv_dtb[cj], c, __fma_rn(w1, Bt[o], -__dmul_rn(w0, Bt[o - G.LD])));
+      e = __fma_rn(id2, k, e);
+    }
     if (lossy) { S.epre[2][l] = e; e = __dmul_rn(e, m.keep_n[ri]); }
     S.f[EPH][o] = e;
   }
@@ -95,6 +103,8 @@ __device__ __forceinline__ void b_node(const EnsFieldArg &S, int i, int j) {
   const size_t o = gidx(G, i, j);
   const double er = S.f[ER][o], er_j = S.f[ER][o + 1], et = S.f[ETH][o], et_i = S.f[ETH][o + G.LD];
   const double ep = S.f[EPH][o], ep_j = S.f[EPH][o + 1], ep_i = S.f[EPH][o + G.LD];
+  // B_th on the axis is not updated: 0, or what pic_set_fields left there
+  const double axis_bt = (j == 0 || j == G.nth) && i < G.nr ? S.f[BTH][o] : 0.0;
   double d[3], d2[3], b[3];
   curl_e(m, ri, cj, er, er_j, et, et_i, ep, ep_j, ep_i, d2);
   const bool lossy = S.lossy_i0 >= 0 && i >= S.lossy_i0;
@@ -118,11 +128,12 @@ __device__ __forceinline__ void b_node(const EnsFieldArg &S, int i, int j) {
     S.f[BR][o] = b[0];
     S.bh[0][o] = __dadd_rn(b[0], d2[0]);
   }
-  if (hi && j >= 1 && hj) {  // B_th at (i+1/2, j); zero on the axis
+  if (hi && j >= 1 && hj) {  // B_th at (i+1/2, j)
     S.f[BTH][o] = b[1];
     S.bh[1][o] = __dadd_rn(b[1], d2[1]);
   } else {
-    b[1] = 0.0;
+    b[1] = axis_bt;
+    if (lossy && hi) S.f[BTH][o] = b[1] = __dmul_rn(axis_bt, m.keep_h[ri]);
   }
   if (hi && hj) {  // B_ph at (i+1/2, j+1/2)
     S.f[BPH][o] = b[2];
