@@ -103,11 +103,13 @@ __device__ __forceinline__ void b_node(const EnsFieldArg &S, int i, int j) {
   const size_t o = gidx(G, i, j);
   const double er = S.f[ER][o], er_j = S.f[ER][o + 1], et = S.f[ETH][o], et_i = S.f[ETH][o + G.LD];
   const double ep = S.f[EPH][o], ep_j = S.f[EPH][o + 1], ep_i = S.f[EPH][o + G.LD];
-  // B_th on the axis is not updated: 0, or what pic_set_fields left there
-  const double axis_bt = (j == 0 || j == G.nth) && i < G.nr ? S.f[BTH][o] : 0.0;
+  // B_th on the axis is not updated: 0, or what pic_set_fields left there, with
+  // its FP32 copy; only the lossy layer changes them
+  const bool lossy = S.lossy_i0 >= 0 && i >= S.lossy_i0;
+  const bool axis = (j == 0 || j == G.nth) && lossy && i < G.nr;
+  const double axis_bt = axis ? S.f[BTH][o] : 0.0;
   double d[3], d2[3], b[3];
   curl_e(m, ri, cj, er, er_j, et, et_i, ep, ep_j, ep_i, d2);
-  const bool lossy = S.lossy_i0 >= 0 && i >= S.lossy_i0;
   if (lossy) {  // the half step before the layer: E as it was then
     const size_t l = (size_t)(i - S.lossy_i0) * G.LD + cj;
     const bool up = i < G.nr;
@@ -131,9 +133,8 @@ __device__ __forceinline__ void b_node(const EnsFieldArg &S, int i, int j) {
   if (hi && j >= 1 && hj) {  // B_th at (i+1/2, j)
     S.f[BTH][o] = b[1];
     S.bh[1][o] = __dadd_rn(b[1], d2[1]);
-  } else {
-    b[1] = axis_bt;
-    if (lossy && hi) S.f[BTH][o] = b[1] = __dmul_rn(axis_bt, m.keep_h[ri]);
+  } else if (axis) {
+    S.f[BTH][o] = b[1] = __dmul_rn(axis_bt, m.keep_h[ri]);
   }
   if (hi && hj) {  // B_ph at (i+1/2, j+1/2)
     S.f[BPH][o] = b[2];
@@ -145,7 +146,8 @@ __device__ __forceinline__ void b_node(const EnsFieldArg &S, int i, int j) {
   if (FP32) {
     q[0] = f64_to_f32(er); q[1] = f64_to_f32(et); q[2] = f64_to_f32(ep);
     q[3] = f64_to_f32(b[0]); q[4] = f64_to_f32(b[1]); q[5] = f64_to_f32(b[2]);
-    S.f32[ER][o] = q[0]; S.f32[EPH][o] = q[2]; S.f32[BTH][o] = q[4];
+    S.f32[ER][o] = q[0]; S.f32[EPH][o] = q[2];
+    if ((hi && j >= 1 && hj) || axis) S.f32[BTH][o] = q[4];
     if (hj) { S.f32[ETH][o] = q[1]; S.f32[BR][o] = q[3]; S.f32[BPH][o] = q[5]; }
   }
   if (j == 0 || j == G.nth - 1) {
